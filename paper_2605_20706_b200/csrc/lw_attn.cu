@@ -9,6 +9,7 @@
 // caller's workspace and a second small kernel merges the parts.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 
@@ -759,18 +760,6 @@ __global__ void __launch_bounds__(288, 1) attn_decode_mma_kernel(const AttnMmaPa
     }
 }
 
-int sm_count_of_current_device() {
-    static int cached[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    if (cached[dev] == 0) {
-        int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
-        cached[dev] = n;
-    }
-    return cached[dev];
-}
-
 template <class Fmt>
 cudaError_t launch_general(const AttnParams& p, cudaStream_t stream) {
     const int nrep_t = p.n_rep <= 1 ? 1 : p.n_rep <= 2 ? 2 : 4;
@@ -830,13 +819,20 @@ int attn_bank_conflicts(int kfmt, bool keys, int row_bytes, int group_stride) {
 }
 
 // Group stride (bytes) with the fewest bank conflicts: the group's rows plus 0..7 pieces of 16 bytes.
+// The simulation takes tens of microseconds, so its answers are kept: one word per format, tensor and row length (a
+// multiple of 16 bytes up to kMaxRowBytes), written with the same value by whichever thread comes first.
+constexpr int kMaxRowBytes = 8192;
 int attn_group_stride(int kfmt, bool keys, int row_bytes) {
+    static std::atomic<int> kept[3][2][kMaxRowBytes / 16 + 1];
+    std::atomic<int>& slot = kept[kfmt][keys ? 1 : 0][row_bytes / 16];
+    if (const int known = slot.load(std::memory_order_relaxed)) return known;
     const int G = attn_group_rows(kfmt);
     int best = G * row_bytes, best_cost = 1 << 30;
     for (int pad = 0; pad < 8; ++pad) {
         const int cost = attn_bank_conflicts(kfmt, keys, row_bytes, G * row_bytes + 16 * pad);
         if (cost < best_cost) best_cost = cost, best = G * row_bytes + 16 * pad;
     }
+    slot.store(best, std::memory_order_relaxed);
     return best;
 }
 
@@ -847,7 +843,7 @@ MmaPlan make_mma_plan(int fmt, int64_t n_head, int64_t n_kv_head, int64_t head_d
     if (n_rep > 64 || (head_dim != 64 && head_dim != 128)) return pl;
     if (n_kv_head != 1 && n_kv_head != 2 && n_kv_head != 4 && n_kv_head != 8) return pl;
     const int64_t rb = (int64_t)lw_row_bytes(fmt, n_kv_head * head_dim);
-    if (rb == 0 || rb % 16 != 0 || rb > 8192) return pl;
+    if (rb == 0 || rb % 16 != 0 || rb > kMaxRowBytes) return pl;
     AttnMmaParams& p = pl.p;
     p.row_bytes = (int)rb;
     const int kfmt = fmt == LW_F16 ? kFmtF16 : fmt == LW_Q8_0 ? kFmtQ8 : kFmtQ4;
@@ -931,7 +927,7 @@ int attn_parts(int64_t n_head, int64_t n_kv_head, int64_t head_dim, int64_t n_po
     const int64_t n_rep = n_head / n_kv_head;
     const int nrep_t = n_rep <= 1 ? 1 : n_rep <= 2 ? 2 : 4;
     (void)head_dim;
-    return general_parts(n_kv_head, (n_rep + nrep_t - 1) / nrep_t, n_pos, sm_count_of_current_device());
+    return general_parts(n_kv_head, (n_rep + nrep_t - 1) / nrep_t, n_pos, device_sm_count());
 }
 
 int64_t attn_workspace_bytes(int64_t n_head, int64_t n_kv_head, int64_t head_dim, int64_t n_pos) {
@@ -943,14 +939,14 @@ void set_attn_variant(int variant) { attn_variant_storage() = variant; }
 
 int attn_variant_of(int fmt, int64_t n_head, int64_t n_kv_head, int64_t head_dim, int64_t n_pos) {
     if (attn_variant_storage() == 1) return 1;
-    return make_mma_plan(fmt, n_head, n_kv_head, head_dim, n_pos, sm_count_of_current_device()).ok ? 2 : 1;
+    return make_mma_plan(fmt, n_head, n_kv_head, head_dim, n_pos, device_sm_count()).ok ? 2 : 1;
 }
 
 int launch_attn_decode(int fmt, const void* K, const void* V, const float* q, float* out, int64_t n_head,
                        int64_t n_kv_head, int64_t head_dim, int64_t n_pos, float scale, void* workspace,
                        cudaStream_t stream) {
     if (attn_variant_storage() != 1) {
-        MmaPlan pl = make_mma_plan(fmt, n_head, n_kv_head, head_dim, n_pos, sm_count_of_current_device());
+        MmaPlan pl = make_mma_plan(fmt, n_head, n_kv_head, head_dim, n_pos, device_sm_count());
         if (pl.ok) {
             pl.p.K = static_cast<const uint8_t*>(K);
             pl.p.V = static_cast<const uint8_t*>(V);

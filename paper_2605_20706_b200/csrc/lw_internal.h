@@ -84,6 +84,8 @@ void set_attn_variant(int variant);
 int attn_variant_of(int fmt, int64_t n_head, int64_t n_kv_head, int64_t head_dim, int64_t n_pos);
 // Address of the per-device fault word (device memory), or nullptr on error.
 int* device_fault_word();
+// SMs of the current device (148 when it cannot be told).
+int device_sm_count();
 
 // Host <-> device copies of a chain's input and result blocks, in pieces that overlap with the chain's kernels
 // (lw_hostpipe.cu).  The chain code calls begin() first, before(j, n) ahead of the launch that runs items

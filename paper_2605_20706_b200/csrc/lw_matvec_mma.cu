@@ -43,6 +43,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "lw.h"
@@ -1270,11 +1271,18 @@ bool make_weight_map(CUtensorMap* map, int fmt, const void* W, int64_t rows, int
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int mma_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    return n;
+// Address of the grid barrier's words on the current device, looked up once per device.
+unsigned* grid_barrier_words() {
+    static std::atomic<unsigned*> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    const bool known = dev >= 0 && dev < 64;
+    if (known)
+        if (unsigned* c = cached[dev].load(std::memory_order_relaxed)) return c;
+    unsigned* p = nullptr;
+    if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_mma_grid_barrier) != cudaSuccess) return nullptr;
+    if (known) cached[dev].store(p, std::memory_order_relaxed);
+    return p;
 }
 
 // Shared-memory plan of a launch: the largest chunk (1024, 512, 256 columns) that divides cols and leaves room
@@ -1363,8 +1371,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
             self_clear = false;
     }
     unsigned* grid_bar = nullptr;
-    if (self_clear && cudaGetSymbolAddress(reinterpret_cast<void**>(&grid_bar), g_mma_grid_barrier) != cudaSuccess)
-        return (int)cudaErrorInvalidValue;
+    if (self_clear && !(grid_bar = grid_barrier_words())) return (int)cudaErrorInvalidValue;
     // the kernel adds every (chunk, row stage) share into Y: clear it first (Y is 16-byte aligned)
     if (!self_clear && !pre_cleared) {
         ZeroList z{};
@@ -1377,7 +1384,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         z.n_items = n_items;
         int64_t blocks = (most / 4 + 255) / 256;
         if (blocks < 1) blocks = 1;
-        if (blocks > 4 * mma_sm_count()) blocks = 4 * mma_sm_count();
+        if (blocks > 4 * device_sm_count()) blocks = 4 * device_sm_count();
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)blocks);
         cfg.blockDim = dim3(256);
@@ -1426,7 +1433,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
     p.w_off = (uint32_t)((kMmaHeader + x_bytes + extra_bytes + w_align - 1) / w_align * w_align);
     const size_t smem_bytes = p.w_off + (size_t)p.ring * stage_bytes;
     const int64_t n_stages = (cols / kStageCols) * (int64_t)rs;
-    int grid = kCtasPerSm * mma_sm_count();
+    int grid = kCtasPerSm * device_sm_count();
     if ((int64_t)grid > n_stages && !self_clear) grid = (int)n_stages;   // self-clearing: every SM, so launches never overlap
     p.drop_stage = -1;
     p.n_next = n_next;

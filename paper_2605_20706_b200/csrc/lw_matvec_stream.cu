@@ -35,10 +35,30 @@ namespace lw {
 
 __device__ int g_fault_word = 0;
 
+// Looked up once per device: the symbol lookup takes a lock and costs a good part of a microsecond, on every launch.
 int* device_fault_word() {
+    static std::atomic<int*> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    const bool known = dev >= 0 && dev < 64;
+    if (known)
+        if (int* c = cached[dev].load(std::memory_order_relaxed)) return c;
     int* p = nullptr;
     if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_fault_word) != cudaSuccess) return nullptr;
+    if (known) cached[dev].store(p, std::memory_order_relaxed);
     return p;
+}
+
+int device_sm_count() {
+    static std::atomic<int> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    int n = cached[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+        cached[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 namespace {
@@ -527,18 +547,6 @@ struct Plan {
     bool ok;
 };
 
-int sm_count() {
-    static int cached[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    if (cached[dev] == 0) {
-        int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        cached[dev] = n;
-    }
-    return cached[dev];
-}
-
 // Launch heuristics [paper Sec 3.2: tunable work-group, tile and per-thread sizes chosen from a
 // sweep].  Tunables: CTAs per SM, ring depth and bytes per ring stage.  The defaults below come
 // from a sweep on B200 over the Llama-shaped matrices; the environment variables LW_CTAS_PER_SM,
@@ -821,7 +829,7 @@ void set_stream_tuning(int worker_groups, int stages, int stage_kb) {
 // Geometry the launch heuristics pick for a shape under the current tuning (for reports).
 bool stream_plan_info(int fmt, int64_t rows, int64_t cols, int* groups, int* stages, int* stage_rows, int* stage_bytes,
                       int* grid, int* smem_bytes) {
-    const Plan pl = make_plan(fmt, true, rows, cols, sm_count());
+    const Plan pl = make_plan(fmt, true, rows, cols, device_sm_count());
     if (!pl.ok) return false;
     *groups = pl.groups;
     *stages = pl.p.stages;
@@ -850,7 +858,7 @@ int launch_matvec_stream_group(int fmt, bool integer_dot, int64_t cols, int n_it
     if (n_items < 1 || n_items > kMaxGroup) return (int)cudaErrorInvalidValue;
     int64_t total_rows = 0;
     for (int j = 0; j < n_items; ++j) total_rows += rows[j];
-    Plan pl = make_plan(fmt, integer_dot, total_rows, cols, sm_count());     // geometry for the whole group
+    Plan pl = make_plan(fmt, integer_dot, total_rows, cols, device_sm_count());     // geometry for the whole group
     if (!pl.ok) return (int)cudaErrorInvalidValue;
     int* fault = device_fault_word();
     if (!fault) return (int)cudaErrorInvalidValue;
@@ -910,7 +918,7 @@ int launch_matvec_stream_batched(int fmt, const void* W, int64_t rows, int64_t c
     if (!fault) return (int)cudaErrorInvalidValue;
     for (int b0 = 0; b0 < batch; b0 += nb_max) {
         const int nb = batch - b0 < nb_max ? batch - b0 : nb_max;
-        Plan pl = make_plan_batched(fmt, rows, cols, nb <= 2 ? 2 : 4, sm_count());
+        Plan pl = make_plan_batched(fmt, rows, cols, nb <= 2 ? 2 : 4, device_sm_count());
         if (!pl.ok) return (int)cudaErrorInvalidValue;
         pl.p.W = static_cast<const uint8_t*>(W);
         pl.p.X = X + (int64_t)b0 * cols;
@@ -931,7 +939,7 @@ int launch_matvec_stream_batched(int fmt, const void* W, int64_t rows, int64_t c
 
 int launch_matvec_stream(int fmt, bool integer_dot, const void* W, int64_t rows, int64_t cols, const float* X,
                          float* Y, bool overlap, cudaStream_t stream) {
-    Plan pl = make_plan(fmt, integer_dot, rows, cols, sm_count());
+    Plan pl = make_plan(fmt, integer_dot, rows, cols, device_sm_count());
     if (!pl.ok) return (int)cudaErrorInvalidValue;
     int* fault = device_fault_word();
     if (!fault) return (int)cudaErrorInvalidValue;
