@@ -13,6 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "liblw.so")
+PYCALL = os.path.join(HERE, "_lwcall.so")          # CPython extension behind the binding's per-call functions
 
 SOURCES = ["lw_matvec_stream.cu", "lw_matvec_seq.cu", "lw_matvec_tile.cu", "lw_matvec_mma.cu", "lw_probe.cu", "lw_attn.cu", "lw_api.cu", "lw_hostpipe.cu", "lw_dequant.cu", "lw_matvec_generic.cu", "lw_quantize.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -27,11 +28,22 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYCALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "lw.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_pycall() -> None:
+    import sysconfig
+    tmp = PYCALL + ".tmp.%d" % os.getpid()
+    proc = subprocess.run(["gcc", "-O2", "-std=c11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "lw_pycall.c"), "-o", tmp], capture_output=True, text=True)
+    if proc.returncode != 0:
+        sys.stderr.write(proc.stdout + proc.stderr)
+        raise RuntimeError("gcc failed on lw_pycall.c")
+    os.replace(tmp, PYCALL)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -67,6 +79,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(link.stdout + link.stderr)
             raise RuntimeError("nvcc failed linking liblw.so")
         os.replace(tmp, LIB)
+        _build_pycall()
     finally:
         shutil.rmtree(objdir, ignore_errors=True)
     return LIB

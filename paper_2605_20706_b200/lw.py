@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the lw C ABI (``include/lw.h``): argument marshalling only.
+"""Thin binding over the lw C ABI (``include/lw.h``): argument marshalling only, by ctypes, and for the calls a
+decode loop repeats by a small CPython extension (csrc/lw_pycall.c).
 
 Every function has the name and meaning of its C counterpart.  Device buffers are passed as torch
 CUDA tensors (or raw integer addresses); PyTorch is used for device memory and streams, nothing
@@ -34,6 +35,7 @@ EXPORTS = ("lw_block_elems", "lw_block_bytes", "lw_row_bytes", "lw_status_string
            "lw_debug_drop_copy", "lw_matvec_sequence", "lw_matvec_sequence_workspace_bytes", "lw_probe_read", "lw_set_sequence_mode", "lw_matvec_sequence_host", "lw_set_shape_tuning", "lw_clear_shape_tuning")
 
 _lib = None
+_call = None          # the per-call entry points as a CPython extension, bound to the loaded library
 
 
 class LwError(RuntimeError):
@@ -96,6 +98,29 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+def _calls():
+    """The extension module behind the per-call functions (csrc/lw_pycall.c), bound to the library on first use."""
+    global _call
+    if _call is None:
+        L = lib()
+        try:
+            from . import _lwcall
+        except ImportError as e:
+            raise RuntimeError("_lwcall.so is missing beside liblw.so: build it with "
+                               "`python -m paper_2605_20706_b200.build`") from e
+        raw = device = None
+        try:
+            import torch
+            raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        except (ImportError, AttributeError):
+            pass                      # another torch: the public lookup serves every call
+        addr = [ctypes.cast(getattr(L, n), ctypes.c_void_p).value
+                for n in ("lw_matvec", "lw_dequant", "lw_matvec_sequence", "lw_matvec_sequence_batch", "lw_attn_decode")]
+        _lwcall.bind(*addr, lambda: _stream_handle(None), raw, device)
+        _call = _lwcall
+    return _call
+
+
 def _addr(buf) -> int:
     """Raw address of a torch tensor, numpy array or integer."""
     if buf is None:
@@ -150,12 +175,15 @@ def quantize(fmt: int, src: np.ndarray, dst: np.ndarray | None = None) -> np.nda
 
 
 def dequant(fmt: int, W_blocks, n: int, out, stream=None) -> None:
-    _check(lib().lw_dequant(fmt, _addr(W_blocks), n, _addr(out), _stream_handle(stream)), "lw_dequant")
+    rc = (_call or _calls()).dequant(fmt, W_blocks, n, out, stream)
+    if rc:
+        raise LwError(rc, "lw_dequant")
 
 
 def matvec(fmt: int, W_blocks, rows: int, cols: int, X, Y, batch: int = 1, stream=None) -> None:
-    _check(lib().lw_matvec(fmt, _addr(W_blocks), rows, cols, _addr(X), _addr(Y), batch,
-                           _stream_handle(stream)), "lw_matvec")
+    rc = (_call or _calls()).matvec(fmt, W_blocks, rows, cols, X, Y, batch, stream)
+    if rc:
+        raise LwError(rc, "lw_matvec")
 
 
 class GroupItem(ctypes.Structure):
@@ -203,8 +231,9 @@ def matvec_sequence(fmt: int, items, workspace, workspace_bytes: int | None = No
     arr = items if isinstance(items, ctypes.Array) else seq_items(items)
     if workspace_bytes is None:
         workspace_bytes = workspace.numel() * workspace.element_size() if hasattr(workspace, "numel") else 0
-    _check(lib().lw_matvec_sequence(fmt, len(arr), ctypes.cast(arr, ctypes.c_void_p), _addr(workspace),
-                                    workspace_bytes, _stream_handle(stream)), "lw_matvec_sequence")
+    rc = (_call or _calls()).sequence(fmt, len(arr), ctypes.addressof(arr), workspace, workspace_bytes, stream)
+    if rc:
+        raise LwError(rc, "lw_matvec_sequence")
 
 
 SEQ_AUTO, SEQ_PERSISTENT, SEQ_LAUNCHES = 0, 1, 2
@@ -229,8 +258,9 @@ def matvec_sequence_host(fmt: int, items, in_host, in_dev, in_bytes: int, out_de
 def matvec_sequence_batch(fmt: int, items, batch: int, stream=None) -> None:
     """A chain of mat-vecs with `batch` columns each: (W_blocks, rows, cols, X, Y, flags) tuples or seq_items()."""
     arr = items if isinstance(items, ctypes.Array) else seq_items(items)
-    _check(lib().lw_matvec_sequence_batch(fmt, len(arr), ctypes.cast(arr, ctypes.c_void_p), batch, _stream_handle(stream)),
-           "lw_matvec_sequence_batch")
+    rc = (_call or _calls()).sequence_batch(fmt, len(arr), ctypes.addressof(arr), batch, stream)
+    if rc:
+        raise LwError(rc, "lw_matvec_sequence_batch")
 
 
 def matvec_sequence_batch_host(fmt: int, items, batch: int, in_host, in_dev, in_bytes: int, out_dev, out_host,
@@ -272,9 +302,10 @@ def attn_decode(kv_fmt: int, K_blocks, V_blocks, q, out, n_head: int, n_kv_head:
     """out[h] = softmax_t(scale * K[t, g] . q[h]) @ V[:, g] for one query token; device buffers."""
     if workspace_bytes is None:
         workspace_bytes = workspace.numel() * workspace.element_size() if hasattr(workspace, "numel") else 0
-    _check(lib().lw_attn_decode(kv_fmt, _addr(K_blocks), _addr(V_blocks), _addr(q), _addr(out), n_head, n_kv_head,
-                                head_dim, n_pos, ctypes.c_float(scale), _addr(workspace), workspace_bytes,
-                                _stream_handle(stream)), "lw_attn_decode")
+    rc = (_call or _calls()).attn_decode(kv_fmt, K_blocks, V_blocks, q, out, n_head, n_kv_head, head_dim, n_pos, scale,
+                                         workspace, workspace_bytes, stream)
+    if rc:
+        raise LwError(rc, "lw_attn_decode")
 
 
 def attn_decode_static(kv_fmt: int, K_blocks, V_blocks, q, out, n_head: int, n_kv_head: int, head_dim: int,
