@@ -250,3 +250,22 @@ def test_attn_host_side_checks():
     assert L.lw_set_attn_variant(1) == lw.OK and L.lw_set_attn_variant(0) == lw.OK
     assert L.lw_query_attn_variant(lw.Q4_K, 32, 8, 128, 10) == lw.ERR_FORMAT
     assert L.lw_query_attn_variant(lw.Q8_0, 32, 5, 128, 10) == lw.ERR_SHAPE
+
+
+@pytest.mark.parametrize("fmt", list(lw.FORMATS.values()))
+@pytest.mark.parametrize("n", [256, 4096, 4096 + 256, 3 * 4096 - 256, 5 * 4096 + 512])
+def test_quantiser_chunks_give_the_oracles_bytes(fmt, n):
+    # the quantiser works in chunks of 4096 weights, eight weights at a time: sizes around a chunk, blocks of tiny, huge,
+    # equal and signed-zero values
+    rng = np.random.default_rng(1000 * fmt + n)
+    x = (rng.standard_normal((n // 32, 32)) * 0.02).astype(np.float32)
+    x[::5] *= np.exp(rng.uniform(-60, 8, (x[::5].shape[0], 1))).astype(np.float32)
+    x[1::7] = x[1::7, :1]
+    x[2::7, ::2] = -0.0
+    x[3::7] = 0.0
+    x[4::11] *= np.float32(1e-38)
+    np.testing.assert_array_equal(lw.quantize(fmt, x.reshape(-1)), oracle.quantize(fmt, x.reshape(-1)))
+    x[-1, -1] = np.inf
+    with pytest.raises(lw.LwError) as e:
+        lw.quantize(fmt, x.reshape(-1))
+    assert e.value.code == lw.ERR_NONFINITE
