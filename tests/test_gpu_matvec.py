@@ -378,3 +378,23 @@ def test_matvec_group_argument_errors():
         lw.matvec_group(lw.Q8_0, 64, [(w, 4, x, y)] * 9, batch=4)
     assert e.value.code == lw.ERR_SHAPE
     assert L.lw_matvec_group_batch(lw.Q8_0, 64, 1, None, 4, None) == lw.ERR_NULL
+
+
+RAGGED = [(f, r, c) for f in (lw.F16, lw.Q8_0, lw.Q4_0, lw.Q4_1, lw.Q5_0, lw.Q5_1)
+          for r, c in [(1, 32), (7, 96), (149, 288), (301, 2848), (1000, 4128), (77, 8224), (40, 16352)]]
+RAGGED += [(lw.Q6_K, r, c) for r, c in [(1, 256), (9, 512), (149, 3072), (1000, 4352), (70, 12544)]]
+RAGGED += [(lw.Q2_K, r, c) for r, c in [(1, 256), (9, 512), (149, 2816), (1000, 4352), (70, 12544)]]
+
+
+@pytest.mark.parametrize("overlap", [False, True])
+@pytest.mark.parametrize("fmt,rows,cols", RAGGED)
+def test_matvec_of_rows_off_the_16_byte_grid(fmt, rows, cols, overlap):
+    # the widths no streaming kernel takes: rows that end off a 16-byte or 4-byte boundary, a last piece of 32 to 224
+    # columns, rows cut into several chunks (above 4096 columns), fewer rows than CTAs
+    blocks = quantized_weights(fmt, rows, cols, seed=61, tensor_id=fmt, outlier_p=0.01)
+    X = synth.activations(61, rows, 1, cols)
+    y_ref, s_ref = oracle.matvec(fmt, blocks, rows, cols, X, 1, nthreads=4)
+    y = gpu_matvec(fmt, blocks, rows, cols, X, overlap=overlap, repeat=2)
+    check_matvec(y, y_ref, s_ref, "fmt %d %dx%d" % (fmt, rows, cols))
+    X[0, cols // 2] = np.nan                       # every output reads it
+    assert not np.isfinite(gpu_matvec(fmt, blocks, rows, cols, X, overlap=overlap)).any()
