@@ -17,10 +17,10 @@
 // The accuracy is that of the fp32 kernels' contract: |y - y_ref| <= 1e-4 * sum|w x| + 1e-6 with no extra term
 // (q4_0, q8_0; q4_K's sub-block offsets go onto fp32 sums of the activations and bring an extra term back, see MmaQ4K).
 //
-// Why mma.sync and not tcgen05.mma here: the A operand is the decoded weight, which exists only in registers
-// (18- and 34-byte blocks decode to fragments with byte permutes); tcgen05.mma reads A from shared or tensor
-// memory, so every weight would take one more store and a proxy fence, for an N of 8..48 whose tensor time is
-// already far below the decode time.  The warp-level form takes the fragments straight from the decode.
+// Two kernels.  matvec_mma_kernel (mma.sync, described here) takes the fragments straight from the decode; it has every
+// quantised format and up to 16 columns.  matvec_tc_kernel (tcgen05.mma, further down) takes f16 and, up to eight columns,
+// large launches of q4_K, q4_0, q4_1 and q8_0 (takes_tc has the rule and the times): there a masked word of codes is an
+// operand of the product as it is, which is worth the extra store of every weight to tensor memory.
 //
 // Layout of the work.  A stage is 256 rows x 256 columns of weights (36 KB of q4_0, 68 KB of q8_0), brought in
 // by a producer thread with one tiled bulk-tensor copy (the matrix as a 2-D tensor of 32-bit words; rows beyond
@@ -75,7 +75,7 @@ constexpr int kTerms = LW_MMA_TERMS;                  // terms an activation is 
 constexpr int kTabRow = 72;                           // bytes between rows of a warp's scale table: 64 of entries + 8, so the
                                                       // eight rows a warp reads at once (8-byte entries) fall into different banks
 constexpr int kSxBlockBytes = 64;                     // block sums of the activations: [block of 32][16 columns] floats
-constexpr int kMmaHeader = 128;                       // barriers, the stop flag and the grid barrier's generation
+constexpr int kMmaHeader = 256;                       // barriers, the stop flag, the grid barrier's generation, tensor memory
 constexpr uint32_t kGridPolls = 1u << 20;             // polls of the generation word (~0.5 us each) before giving up
 
 // Grid barrier of the self-clearing launches: {count, generation}.  A launch holds every SM (one CTA per SM,
@@ -104,6 +104,9 @@ struct MmaParams {
     MmaItem item[kMmaMaxItems];
     int n_items;
     int total_rs;         // row stages of all matrices
+    int share, extra;     // stages of a CTA; the first `extra` CTAs take one more (64-bit divisions in every warp's prologue
+                          // cost 0.3 us)
+    int spc_shift;        // log2 of the stages per (chunk, row stage)
     int batch;            // columns of this launch (<= 8 NT)
     int chunk_cols;       // 256, 512 or 1024: columns whose activations are resident at a time
     int ring;             // stages in the ring (2..kMaxRing)
@@ -199,7 +202,6 @@ __device__ __forceinline__ uint32_t bytes_to_bf16_128_plus(uint32_t v) {
 // the row's piece of the stage plus 4 t (t = lane % 4), OFF = byte offset of the two-block unit from there.
 struct MmaQ40 {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 8 * 18;               // bytes of a row's 256 columns
@@ -232,7 +234,6 @@ struct MmaQ40 {
 
 struct MmaQ80 {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 8 * 34;
@@ -276,7 +277,6 @@ struct MmaQ80 {
 // accuracy statement).  The 6-bit fields are unpacked once per warp and stage into a table of (d * sc, dmin * m).
 struct MmaQ4K {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 144;
@@ -333,7 +333,6 @@ struct MmaQ4K {
 // s of byte l is the high bit of weight l of sub-block s, so a code is 0..31 -- still exact in bf16.
 struct MmaQ5K {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 176;
@@ -398,7 +397,6 @@ struct MmaLegacy {
     static constexpr bool kHasMin = FMT != LW_Q5_0;
     static constexpr int kBlock = FMT == LW_Q4_1 ? 20 : (FMT == LW_Q5_0 ? 22 : 24);
     static constexpr int kStageRows = 256;
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     // 16 bytes more than a row's 256 columns are fetched for q4_1 and q5_1: their 160- and 192-byte pitches would put
@@ -446,79 +444,6 @@ struct MmaLegacy {
     }
 };
 
-// f16 weights: they are the A operand as they lie in memory (mma with f16 operands), nothing is decoded.  A row's
-// 256 columns are 512 bytes, fetched as four 128-byte slices (one per 64-column unit) with the 128-byte swizzle of
-// the tensor copy, so that the eight rows a warp reads at once fall into different banks: 16-byte chunk c of row r
-// of a slice sits at chunk c ^ (r % 8).  A stage is 128 rows; warps 0-7 take units 0 and 1 of their 16 rows, warps
-// 8-15 units 2 and 3.  The activations are held as f16 terms of x * s, s a power of two per block of 32 and
-// column that brings the block's largest magnitude to 2^14..2^15: the first term is cut off exactly, the second
-// rounds what is left (22 significant bits of the element, but nothing below 2^-38 of the block's largest
-// magnitude: the extra term E of the accuracy statement with a tiny constant); 1 / s multiplies the block's sum.
-struct MmaF16 {
-    static constexpr int kStageRows = 128;
-    static constexpr bool kF16 = true;
-    static constexpr bool kQ6K = false;
-    static constexpr bool kQ2K = false;
-    static constexpr int kPiece = 512;
-    static constexpr bool kHasMin = false;
-    static constexpr int kTableBytes = 0;
-    static constexpr int kSliceBytes = kStageRows * 128;     // one unit of all the stage's rows
-};
-
-__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                        uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_f16_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                              uint32_t b0, uint32_t b1) {
-    asm("{\n\t.reg .f32 z;\n\tmov.f32 z, 0f00000000;\n\t"
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{z, z, z, z};\n\t}"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// One block of 32 f16 weights of the warp's 16 rows against all columns.  wrow = address of row g's 128 bytes in
-// slice 0 of the stage plus 8 (t % 2); sw[h] = byte offset of the lane's swizzled 16-byte chunk for half h of block
-// 0 (block 1: sw[2 + h]); sx = the lane's two block scales (1 / s), group nt 32 bytes further.
-template <int NT, int U, int BLK>
-__device__ __forceinline__ void block_step_f16(uint32_t wrow, const uint32_t (&sw)[4], uint32_t sx,
-                                               const uint32_t (&xp)[NT][kTerms], float (&y)[NT][4]) {
-    constexpr int kSlice = U * MmaF16::kSliceBytes;
-    uint32_t a[4], b[4];
-    lds64<kSlice>(wrow + sw[2 * BLK], a[0], a[1]);               // row g: k = 4t .. 4t+3
-    lds64<kSlice>(wrow + sw[2 * BLK + 1], a[2], a[3]);           //        k = 16+4t ..
-    lds64<kSlice + 8 * 128>(wrow + sw[2 * BLK], b[0], b[1]);     // row g + 8 (same swizzle: (g + 8) % 8 == g)
-    lds64<kSlice + 8 * 128>(wrow + sw[2 * BLK + 1], b[2], b[3]);
-    constexpr int kX = 2 * (64 * U + 32 * BLK);
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        float c[4];
-#pragma unroll
-        for (int s = 0; s < kTerms; ++s) {
-            uint32_t b0, b1, b2, b3;
-            lds128<kX>(xp[nt][s], b0, b1, b2, b3);
-            if (s == 0)
-                mma_f16_first(c, a[0], b[0], a[1], b[1], b0, b1);
-            else
-                mma_f16(c, a[0], b[0], a[1], b[1], b0, b1);
-            mma_f16(c, a[2], b[2], a[3], b[3], b2, b3);
-        }
-        float s0, s1;                                            // 1 / s of columns 2 t and 2 t + 1 of the group
-        if (nt == 0)
-            lds_f32x2<kSxBlockBytes * (2 * U + BLK)>(sx, s0, s1);
-        else
-            lds_f32x2<kSxBlockBytes * (2 * U + BLK) + 32>(sx, s0, s1);
-        y[nt][0] = fmaf(s0, c[0], y[nt][0]);
-        y[nt][1] = fmaf(s1, c[1], y[nt][1]);
-        y[nt][2] = fmaf(s0, c[2], y[nt][2]);
-        y[nt][3] = fmaf(s1, c[3], y[nt][3]);
-    }
-}
-
 // q6_K: 210-byte super-blocks {128 bytes of low nibbles, 64 bytes of upper bit pairs, 16 int8 scales (one per 16
 // weights), d}.  210 is not a multiple of 16, so a row's piece of a stage starts anywhere on a 2-byte grid: the
 // tensor copy starts at the 16-byte boundary below it and fetches 240 bytes per row, and the kernel indexes from
@@ -529,7 +454,6 @@ __device__ __forceinline__ void block_step_f16(uint32_t wrow, const uint32_t (&s
 // bytes l and l + 32) for even U and {2, 3} (high nibbles) for odd U.
 struct MmaQ6K {
     static constexpr int kStageRows = 256;
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = true;
     static constexpr bool kQ2K = false;
     static constexpr int kSuper = 210;                  // bytes of 256 weights
@@ -558,7 +482,6 @@ struct MmaQ6K {
 // sums of each 16 activations (extra term E, c = 2^-18).  Unit U = half U / 2, groups {0, 1} or {2, 3}.
 struct MmaQ2K {
     static constexpr int kStageRows = 256;
-    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = true;
     static constexpr int kSuper = 84;
@@ -792,18 +715,189 @@ __device__ __forceinline__ void split3(float x, uint32_t& h1, uint32_t& h2, uint
     }
 }
 
-// fp32 -> f16 terms of x (already scaled into the f16 range): cut off (exact differences) except the last, which
-// rounds the rest
-__device__ __forceinline__ void split3_f16(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
-    unsigned short a, b, c;
-    asm("cvt.rz.f16.f32 %0, %1;" : "=h"(a) : "f"(x));
-    const float r1 = x - __half2float(__ushort_as_half(a));
-    if (kTerms == 2) asm("cvt.rn.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
-    else asm("cvt.rz.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
-    const float r2 = r1 - __half2float(__ushort_as_half(b));
-    asm("cvt.rn.f16.f32 %0, %1;" : "=h"(c) : "f"(r2));
-    h1 = a, h2 = b, h3 = c;
+// ------------------------------------------------------------------ tcgen05 kernel ---
+//
+// A lane owns one ROW: it reads the row's codes of 128 columns with 16-byte shared-memory loads (row pitches are odd
+// multiples of 16 bytes: conflict-free), turns them into bf16 numbers and stores them to tensor memory, where lane r of
+// the A operand is row r.  One thread per pair of warpgroups issues the products (M = 128 rows, N = 16, K = 16 per
+// instruction: 9.2 clocks each, measured) with the activations as the B operand in shared memory, one accumulator per block
+// of 32 weights, and the lane reads its row's sums back and applies the block scales in fp32.
+//
+// Decoding costs almost nothing: the bf16 with the integer u <= 255 as its bit pattern IS the number u * 2^-133 (seven bits
+// subnormal, the eighth the lowest exponent bit; the tensor core multiplies such numbers exactly), so masking a word with
+// 0x000F000F gives two nibbles ready to multiply, 0x00F000F0 two nibbles times 16, and one packed addition takes q4_0's
+// 8 or q8_0's 128 off.  Up to 8 columns about 210 warp instructions per 2048 4-bit weights (decode and stores to tensor
+// memory 80, reading the sums back and scaling 55, the rest waits and loop), against 257 for the warp-level form (one
+// byte permute and one subtraction per pair of weights, fragments of two rows per lane, scale tables): that is the bound,
+// 56 % of the issue slots; the tensor pipe is busy a fifth of the time.
+//
+// B: bf16 terms of x * s, s the power of two that brings the largest magnitude of 128 columns to 2^126..2^127, which with the
+// 2^-133 of the codes leaves products in the middle of fp32's range: no term is lost down to 2^-120 of the largest, and the
+// accuracy is that of the warp-level form (two terms, 2^-16 of each element).  q4_0, q4_1: x / 16 for the upper nibbles.
+// q4_K's offsets: one more product, of their codes with the sums of the blocks' activations as three terms (exact).
+// f16 weights: A as it lies in memory, B two f16 terms of x * s, s per block of 32 columns (largest to 2^14..2^15: 22
+// significant bits, but nothing below 2^-38 of the block's largest).
+// Layout of B: [k / 8][16 n][8 k], n = 8 term + column (9 to 16 columns: a plane per term), 272 bytes per group of 8 k (16
+// of padding: the conversion's stores fall into different banks).  Inside each four k the order is 0, 2, 1, 3 (kQuad), as the
+// masks give.
+
+__device__ __forceinline__ uint4 lds_v4(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
 }
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// 16-byte pieces of a row that cover bytes [B, B + N), B and N known at compile time; word(off) = the 32-bit word at byte
+// off of the row (2-byte aligned), half(off) = the f16 there.
+template <int B, int N>
+struct RowBytes {
+    static constexpr int kFirst = B & ~15, kPieces = (B + N - kFirst + 15) / 16;
+    uint32_t w[4 * kPieces];
+    __device__ __forceinline__ void load(uint32_t row) {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const uint4 v = lds_v4(row + kFirst + 16 * i);
+            w[4 * i] = v.x, w[4 * i + 1] = v.y, w[4 * i + 2] = v.z, w[4 * i + 3] = v.w;
+        }
+    }
+    __device__ __forceinline__ uint32_t word(int off) const {
+        const int i = (off - kFirst) >> 2;
+        return (off & 2) ? __byte_perm(w[i], w[i + 1], 0x5432u) : w[i];
+    }
+    __device__ __forceinline__ float half(int off) const {
+        const uint32_t v = w[(off - kFirst) >> 2];
+        return __half2float(__ushort_as_half((unsigned short)((off & 2) ? v >> 16 : v & 0xFFFFu)));
+    }
+};
+// byte i (compile time) of v times d: (2^23 + byte) * d - 2^23 d, exactly
+__device__ __forceinline__ float byte_times(uint32_t v, int i, float d, float nd) {
+    return fmaf(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7440u | i)), d, nd);
+}
+
+// Traits: G = which 64 columns of the stage's 256.  frag(a): those as 32 words of two bf16 numbers, in the K order of the
+// tensor core.  scales(d): factors of the sums of its two blocks, times 2^24.  Formats with an offset per block: offset(m) =
+// the offsets; kMinProduct formats instead mins() = the two blocks' offset codes as bf16 numbers -- they are multiplied with
+// the sums of the blocks' activations, one more product of the tensor core -- and min_factor() = the factor of that result.
+template <int FMT>
+struct TcLegacy {
+    static constexpr bool kEight = FMT == LW_Q8_0;
+    static constexpr bool kHasMin = FMT == LW_Q4_1, kMinProduct = false;
+    static constexpr int kBlock = kEight ? 34 : 18 + (kHasMin ? 2 : 0);
+    static constexpr int kStageRows = 256;
+    static constexpr bool kF16 = false;
+    static constexpr bool kQuad = true;                 // K order 0, 2, 1, 3 inside four
+    static constexpr bool kUpperScaled = !kEight;       // the upper 16 weights of a block come as 16 * code: B holds x / 16 for them
+    static constexpr int kPiece = 8 * kBlock + (kHasMin ? 16 : 0);     // (160 is an even multiple of 16)
+    static constexpr int kXWords = 8 * kBlock / 4;
+    template <int G>
+    struct Row {
+        RowBytes<2 * kBlock * G, 2 * kBlock> b;
+        __device__ __forceinline__ void load(uint32_t row) { b.load(row); }
+        __device__ __forceinline__ void frag(uint32_t (&a)[32]) const {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int q = kBlock * (2 * G + j) + 2 + (kHasMin ? 2 : 0);
+                if constexpr (kEight) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        // the byte code + 128, minus 128
+                        const uint32_t x = b.word(q + 4 * i) ^ 0x80808080u;
+                        a[16 * j + 2 * i] = add_bf16x2(__byte_perm(x, 0u, 0x4240u), 0x80808080u);
+                        a[16 * j + 2 * i + 1] = add_bf16x2(__byte_perm(x, 0u, 0x4341u), 0x80808080u);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t w = b.word(q + 4 * i), v = w >> 8;
+                        uint32_t e[4] = {w & 0x000F000Fu, v & 0x000F000Fu, w & 0x00F000F0u, v & 0x00F000F0u};
+                        if constexpr (!kHasMin) {                  // -8, resp. -8 * 16
+                            e[0] = add_bf16x2(e[0], 0x80088008u), e[1] = add_bf16x2(e[1], 0x80088008u);
+                            e[2] = add_bf16x2(e[2], 0x80808080u), e[3] = add_bf16x2(e[3], 0x80808080u);
+                        }
+                        a[16 * j + 2 * i] = e[0], a[16 * j + 2 * i + 1] = e[1];
+                        a[16 * j + 8 + 2 * i] = e[2], a[16 * j + 8 + 2 * i + 1] = e[3];
+                    }
+                }
+            }
+        }
+        __device__ __forceinline__ void scales(float* d) const {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) d[u] = b.half(kBlock * (2 * G + u)) * 16777216.f;
+        }
+        __device__ __forceinline__ void offset(float* m) const {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) m[u] = kHasMin ? b.half(kBlock * (2 * G + u) + 2) : 0.f;
+        }
+    };
+};
+
+struct TcK4 {
+    static constexpr bool kHasMin = true, kMinProduct = true, kF16 = false, kQuad = true, kUpperScaled = false;
+    static constexpr int kStageRows = 256;
+    static constexpr int kPiece = 144, kXWords = kPiece / 4;
+    template <int G>
+    struct Row {
+        uint4 head;
+        RowBytes<16 + 32 * G, 32> b;
+        __device__ __forceinline__ void load(uint32_t row) {
+            head = lds_v4(row);
+            b.load(row);
+        }
+        __device__ __forceinline__ void frag(uint32_t (&a)[32]) const {
+            // the low nibbles of the 32 bytes are sub-block 2 G, the high ones (16 q) the next
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t w = b.w[i], v = w >> 8;
+                a[2 * i] = w & 0x000F000Fu, a[2 * i + 1] = v & 0x000F000Fu;
+                a[16 + 2 * i] = w & 0x00F000F0u, a[16 + 2 * i + 1] = v & 0x00F000F0u;
+            }
+        }
+        static constexpr int kAt = 2 * (G & 1);                   // byte of sub-block 2 G in its half's fields
+        __device__ __forceinline__ void scales(float* d) const {
+            const uint32_t sc = G < 2 ? head.y & 0x3F3F3F3Fu : (head.w & 0x0F0F0F0Fu) | ((head.y >> 2) & 0x30303030u);
+            const float dd = half_lo_to_float(head.x);
+            const float d0 = dd * 16777216.f, d1 = dd * 1048576.f;       // (the second block's codes are 16 q)
+            d[0] = byte_times(sc, kAt, d0, -8388608.f * d0), d[1] = byte_times(sc, kAt + 1, d1, -8388608.f * d1);
+        }
+        __device__ __forceinline__ uint32_t mins() const {
+            const uint32_t mn = G < 2 ? head.z & 0x3F3F3F3Fu : ((head.w >> 4) & 0x0F0F0F0Fu) | ((head.z >> 2) & 0x30303030u);
+            return __byte_perm(mn, 0u, kAt == 0 ? 0x4140u : 0x4342u);
+        }
+        __device__ __forceinline__ float min_factor() const { return -16777216.f * half_hi_to_float(head.x); }
+    };
+};
+
+// f16 weights are the A operand as they lie in memory.  A stage is 128 rows, fetched as four 128-byte slices per row (64
+// columns each, one per warpgroup) with the 128-byte swizzle: 16-byte chunk c of row r sits at chunk c ^ (r % 8).
+struct TcF16 {
+    static constexpr bool kHasMin = false, kMinProduct = false, kF16 = true, kQuad = false, kUpperScaled = false;
+    static constexpr int kStageRows = 128, kPiece = 512, kXWords = 0;
+    static constexpr int kSliceBytes = kStageRows * 128;
+    template <int G>
+    struct Row {};
+};
+
+// Two activations (already scaled) as two terms each, packed (x0 low): the first cut off (exact difference), the second
+// rounds the rest
+template <bool F16>
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& h1, uint32_t& h2) {
+    if constexpr (F16) {
+        unsigned short a, b;
+        asm("cvt.rz.f16.f32 %0, %1;" : "=h"(a) : "f"(x0));
+        asm("cvt.rz.f16.f32 %0, %1;" : "=h"(b) : "f"(x1));
+        h1 = a | ((uint32_t)b << 16);
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h2) : "f"(x1 - __half2float(__ushort_as_half(b))), "f"(x0 - __half2float(__ushort_as_half(a))));
+    } else {
+        const uint32_t a = __float_as_uint(x0) & 0xFFFF0000u, b = __float_as_uint(x1) & 0xFFFF0000u;
+        h1 = __byte_perm(a, b, 0x7632u);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h2) : "f"(x1 - __uint_as_float(b)), "f"(x0 - __uint_as_float(a)));
+    }
+}
+constexpr int kInvBytes = 32 * 64;              // 1 / s of the activations: [run of the chunk][16 columns] floats
 
 // Clears the Y of every matrix of a launch of the kernel below.  Launched like it (see launch_matvec_mma_group): lets
 // its successor start its set-up at once and waits for its predecessor before it writes.
@@ -831,11 +925,11 @@ __global__ void __launch_bounds__(256) zero_kernel(const __grid_constant__ ZeroL
 struct Cursor {
     int c, rs, j, slot, it;
     uint32_t parity;
-    __device__ __forceinline__ void init(const MmaParams& p, int64_t first, int spc) {
-        const int64_t pair = first / spc;
-        j = (int)(first - pair * spc);
-        c = (int)(pair / p.total_rs);
-        rs = (int)(pair - (int64_t)c * p.total_rs);
+    __device__ __forceinline__ void init(const MmaParams& p, unsigned first, int spc) {
+        const unsigned pair = first >> p.spc_shift;
+        j = (int)(first & (unsigned)(spc - 1));
+        c = (int)(pair / (unsigned)p.total_rs);
+        rs = (int)(pair - (unsigned)c * (unsigned)p.total_rs);
         it = 0;
         while (it + 1 < p.n_items && rs >= p.item[it + 1].rs_begin) ++it;
         slot = 0;
@@ -877,11 +971,9 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
     const int Kx = p.chunk_cols;
     const uint32_t x_pitch = 2u * Kx + kXPad;                         // bytes between columns of a plane
     const uint32_t plane_pitch = NB * x_pitch;
-    const int spc = Kx / kStageCols;                                  // stages per (chunk, row stage)
-    const int n_rs = p.total_rs;
-    const int n_chunks = (int)(p.cols / Kx);
-    const int64_t n_stages = (int64_t)n_chunks * n_rs * spc;
-    const int64_t first = n_stages * blockIdx.x / gridDim.x, last = n_stages * (blockIdx.x + 1) / gridDim.x;
+    const int spc = 1 << p.spc_shift;                                 // stages per (chunk, row stage)
+    const unsigned first = (unsigned)p.share * blockIdx.x + min(blockIdx.x, (unsigned)p.extra);
+    const unsigned last = first + (unsigned)p.share + (blockIdx.x < (unsigned)p.extra ? 1u : 0u);
     const int ring = p.ring;
 
     // With programmatic dependent launch this kernel may have been placed while its predecessor on the stream
@@ -920,14 +1012,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                 break;
             }
             mbar_expect_tx(&full[cur.slot], kStageBytes);   // a box always delivers all its bytes (zeros past the end)
-            if constexpr (T::kF16) {
-                // four swizzled 128-byte slices (one per 64-column unit), each all the stage's rows
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    tensor_load_2d(smem + p.w_off + (size_t)cur.slot * kStageBytes + u * MmaF16::kSliceBytes,
-                                   &maps.m[cur.it], ((cur.c * spc + cur.j) * 4 + u) * 32,
-                                   (cur.rs - p.item[cur.it].rs_begin) * kStageRows, &full[cur.slot], policy);
-            } else if constexpr (T::kQ6K || T::kQ2K) {
+            if constexpr (T::kQ6K || T::kQ2K) {
                 // the piece starts at byte kSuper * (stage's column index) of the row: fetch from the 16-byte boundary below
                 tensor_load_2d(smem + p.w_off + (size_t)cur.slot * kStageBytes, &maps.m[cur.it],
                                ((T::kSuper * (cur.c * spc + cur.j)) >> 4) << 2,
@@ -979,13 +1064,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
     const uint32_t xs = smem_u32(smem + p.x_off);
     // this lane's B fragments: column g of each group of eight, slots 8 t .. 8 t + 7 of a block of 32
     const uint32_t xlane = xs + g * x_pitch + 16u * t;
-    // the warp's 16 rows of a stage; f16: 128-row stages, warps 0-7 take units 0 and 1, warps 8-15 units 2 and 3
-    const int mt = T::kF16 ? (warp & 7) : warp;
-    const uint32_t wrow = smem_u32(smem + p.w_off) +
-                          (T::kF16 ? (uint32_t)(16 * mt + g) * 128u + 8u * (t & 1) : (uint32_t)(16 * warp + g) * kPiece);
-    uint32_t sw[4];                                     // f16: the lane's swizzled chunk offsets (see block_step_f16)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) sw[i] = (uint32_t)(((2 * i + (t >> 1)) ^ g) << 4);
+    const uint32_t wrow = smem_u32(smem + p.w_off) + (uint32_t)(16 * warp + g) * kPiece;      // the warp's 16 rows of a stage
 
     float y[NT][4];
 #pragma unroll
@@ -1014,7 +1093,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             cleared = true;
         }
         const MmaItem& m = p.item[cur_it];
-        const int64_t r = (int64_t)(cur_rs - m.rs_begin) * kStageRows + 16 * mt + g;
+        const int64_t r = (int64_t)(cur_rs - m.rs_begin) * kStageRows + 16 * warp + g;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -1038,7 +1117,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             cur_it = cur.it;
         }
         if (c != cur_c || mat.X != cur_x) {
-            // the chunk's activations as one bf16 (f16) plane per term: plane s, column b.  Inside a block of 32 the order is
+            // the chunk's activations as one bf16 plane per term: plane s, column b.  Inside a block of 32 the order is
             // the one the fragments want: slots 8 q .. 8 q + 3 hold k = 4 q .. 4 q + 3 and slots 8 q + 4 .. 8 q + 7
             // hold k = 16 + 4 q .., so a lane reads both halves of its B operand with one 16-byte load.
             cur_c = c;
@@ -1072,29 +1151,10 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                         const int idx = tid + nt * kMmaComputeThreads;
                         const int b = idx >> 6, k4 = jj * (kStageCols / 4) + (idx & 63);
                         uint32_t h[3][4];
-                        if constexpr (T::kF16) {
-                            // f16 terms of x * s, s = the power of two that brings the block's largest magnitude (eight
-                            // consecutive lanes hold a block of 32) to 2^14 .. 2^15; 1 / s goes to [block][column]
-                            float mx = fmaxf(fmaxf(fabsf(v[q][nt].x), fabsf(v[q][nt].y)), fmaxf(fabsf(v[q][nt].z), fabsf(v[q][nt].w)));
-                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-                            int se = 268 - (int)((__float_as_uint(mx) >> 23) & 0xFFu);      // biased exponent of s
-                            se = se < 1 ? 1 : (se > 253 ? 253 : se);
-                            const float sc = __uint_as_float((uint32_t)se << 23);
-                            if ((lane & 7) == 0)
-                                *reinterpret_cast<float*>(smem + p.sx_off + (size_t)(k4 >> 3) * kSxBlockBytes + 4 * b) =
-                                    __uint_as_float((uint32_t)(254 - se) << 23);
-                            split3_f16(v[q][nt].x * sc, h[0][0], h[1][0], h[2][0]);
-                            split3_f16(v[q][nt].y * sc, h[0][1], h[1][1], h[2][1]);
-                            split3_f16(v[q][nt].z * sc, h[0][2], h[1][2], h[2][2]);
-                            split3_f16(v[q][nt].w * sc, h[0][3], h[1][3], h[2][3]);
-                        } else {
-                            split3(v[q][nt].x, h[0][0], h[1][0], h[2][0]);
-                            split3(v[q][nt].y, h[0][1], h[1][1], h[2][1]);
-                            split3(v[q][nt].z, h[0][2], h[1][2], h[2][2]);
-                            split3(v[q][nt].w, h[0][3], h[1][3], h[2][3]);
-                        }
+                        split3(v[q][nt].x, h[0][0], h[1][0], h[2][0]);
+                        split3(v[q][nt].y, h[0][1], h[1][1], h[2][1]);
+                        split3(v[q][nt].z, h[0][2], h[1][2], h[2][2]);
+                        split3(v[q][nt].w, h[0][3], h[1][3], h[2][3]);
                         if constexpr (T::kQ2K) {
                             // sums of each 16 activations (four consecutive lanes hold them): [block][half][column]
                             float sum = (v[q][nt].x + v[q][nt].y) + (v[q][nt].z + v[q][nt].w);
@@ -1132,7 +1192,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             }
         }
         const int64_t r0 = (int64_t)(rs - mat.rs_begin) * kStageRows;
-        if (r0 + 16 * mt < mat.rows) {
+        if (r0 + 16 * warp < mat.rows) {
             const uint32_t row = wrow + (uint32_t)slot * kStageBytes, wt = row + 4u * t;
             const uint32_t tab = smem_u32(smem + p.tab_off) + (uint32_t)warp * T::kTableBytes, tabg = tab + (uint32_t)kTabRow * g;
             const uint32_t sx = smem_u32(smem + p.sx_off) + (uint32_t)(8 * j) * kSxBlockBytes + 8u * t;
@@ -1167,19 +1227,6 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                     stage_q6k<NT, true>(wt + (o & ~3u), tabg, xp, y);
                 else
                     stage_q6k<NT, false>(wt + o, tabg, xp, y);
-            } else if constexpr (T::kF16) {
-                const uint32_t wr = wrow + (uint32_t)slot * kStageBytes;
-                if (warp < 8) {
-                    block_step_f16<NT, 0, 0>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 0, 1>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 1, 0>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 1, 1>(wr, sw, sx, xp, y);
-                } else {
-                    block_step_f16<NT, 2, 0>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 2, 1>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 3, 0>(wr, sw, sx, xp, y);
-                    block_step_f16<NT, 3, 1>(wr, sw, sx, xp, y);
-                }
             } else {
                 block_step<T, NT, 0, 0>(wt, row, tabg, sx, xp, y);
                 block_step<T, NT, 0, 1>(wt, row, tabg, sx, xp, y);
@@ -1203,6 +1250,583 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
         for (int64_t i = q0 + tid; i < q1; i += kMmaComputeThreads) y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (blockIdx.x == 0 && tid < (int)(p.next_n[it] - 4 * quads)) p.next_y[it][4 * quads + tid] = 0.f;
     }
+}
+
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(v));
+    return v;
+}
+// D (tensor memory, 128 x 16 fp32) {+}= A (tensor memory, 128 x 16 f16) * B (shared memory descriptor, 16 x 16 f16)
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool add) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+                 "r"(a), "l"(b), "r"(idesc), "r"((uint32_t)add)
+                 : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_st32(uint32_t t, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, "
+        "%18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(t),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]),
+        "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]),
+        "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+}
+// N consecutive columns of the lane's row.  The registers hold them after the wait below, through which they pass, so
+// that nothing that uses them can be moved in front of it.
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t t, uint32_t* r) {
+    static_assert(N == 4 || N == 8 || N == 16, "");
+    if constexpr (N == 4) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(t));
+    } else if constexpr (N == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(t));
+    } else {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+              "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(t));
+    }
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[N]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
+
+constexpr int kKGroup = 272;                    // bytes of B per eight k: 16 rows of 16 bytes, 16 of padding
+// Tensor-memory columns of a warpgroup: 64 of A, then the accumulators of the four blocks.  With 16 columns of activations these
+// take 16 each.  Up to 8 columns they lie 8 apart although a product writes 16: what it writes into the next one's place is
+// overwritten by that one's own first product (they are issued in order); behind them the accumulator of the offsets,
+// and at 112 the offsets' A operand.
+constexpr uint32_t kRegionCols = 128;
+constexpr uint32_t kMinsCol = 112;
+constexpr int kMinRun = 512;                    // bytes of the offsets' B operand per run of 128 columns: [2][16 n][8 k]
+// instruction descriptor: D fp32, A and B f16 or both bf16 (K major), N = 16, M = 128
+constexpr uint32_t kTcDescF16 = (1u << 4) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kTcDescBf16 = kTcDescF16 | (1u << 7) | (1u << 10);
+
+// y[i] += yp[i] * (the pair i of the floats at shared address at)
+template <int N>
+__device__ __forceinline__ void add_scaled(uint32_t at, const f2 (&yp)[N], f2 (&y)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        f2 s0, s1;
+        asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(s0), "=l"(s1) : "r"(at + 8u * i));
+        y[i] = fma2(yp[i], s0, y[i]);
+        y[i + 1] = fma2(yp[i + 1], s1, y[i + 1]);
+    }
+}
+
+// A CTA's range of stages as runs: consecutive stages of one (chunk, row stage).
+struct RunCursor {
+    int c, rs, it, j, left;            // left: stages of the run (within the CTA's range)
+    __device__ __forceinline__ void init(const MmaParams& p, unsigned first, int spc, int total) {
+        const unsigned pair = first >> p.spc_shift;
+        j = (int)(first & (unsigned)(spc - 1));
+        c = (int)(pair / (unsigned)p.total_rs);
+        rs = (int)(pair - (unsigned)c * (unsigned)p.total_rs);
+        it = 0;
+        while (it + 1 < p.n_items && rs >= p.item[it + 1].rs_begin) ++it;
+        left = min(spc - j, total);
+    }
+    __device__ __forceinline__ void next(const MmaParams& p, int spc, int total_left) {
+        j = 0;
+        left = min(spc, total_left);
+        if (++rs == p.total_rs) rs = 0, it = 0, ++c;
+        else if (it + 1 < p.n_items && rs >= p.item[it + 1].rs_begin) ++it;
+    }
+};
+
+// CB = columns a launch holds: 4, 8 or 16; the terms of a block are added into the same accumulator.
+// T::kStageRows x 256 columns per stage.  Warpgroup wg of the four: quantised formats: rows 128 (wg % 2) .., columns
+// 128 (wg / 2) ..; f16: all 128 rows, columns 64 wg ..
+// A warpgroup's products run while it reads and decodes the first half of its share of the next stage: the compute warps
+// signal "A is in tensor memory", one of two issuing threads (each serves two warpgroups) waits for that, issues and commits
+// to "products complete"; then the warps read the sums back, apply the scales and hand the next A over.
+constexpr int kTcThreads = kMmaComputeThreads + 128;   // the producer warp is in a warpgroup of its own (setmaxnreg)
+// Registers per thread: 640 threads are launched with 96 each; the producer's warpgroup gives most of its share away.
+constexpr int kTcComputeRegs = 112, kTcProducerRegs = 32;
+static_assert(kMmaComputeThreads * kTcComputeRegs + 128 * kTcProducerRegs <= kTcThreads * 96, "register shares exceed the launch's total");
+template <class T, int CB, bool DROP = false>
+__global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_constant__ MmaParams p,
+                                                                  const __grid_constant__ MmaMaps maps) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);               // [kMaxRing]
+    uint64_t* empty = full + kMaxRing;                                // [kMaxRing]
+    volatile int* stop = reinterpret_cast<volatile int*>(smem + 64);  // set when a wait gave up
+    uint64_t* ready = reinterpret_cast<uint64_t*>(smem + 128);        // [4] a warpgroup's A is in tensor memory
+    uint64_t* done = reinterpret_cast<uint64_t*>(smem + 160);         // [4] its products are complete
+    constexpr int kStageBytes = T::kStageRows * T::kPiece;
+    constexpr bool kPlanes = CB == 16;
+    constexpr bool kMinProduct = T::kMinProduct;
+    constexpr uint32_t kTcDesc = T::kF16 ? kTcDescF16 : kTcDescBf16;
+    static_assert(T::kF16 || !kPlanes, "the quantised formats hold up to eight columns");
+    constexpr int kAccStep = kPlanes ? 16 : 8;                        // tensor-memory columns between accumulators
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);           // uniform, for the compiler too
+    const int Kx = p.chunk_cols;
+    const uint32_t plane_bytes = (uint32_t)(Kx / 8) * kKGroup;
+    const int spc = 1 << p.spc_shift;                                 // stages per (chunk, row stage)
+    const unsigned first = (unsigned)p.share * blockIdx.x + min(blockIdx.x, (unsigned)p.extra);
+    const int count = p.share + (blockIdx.x < (unsigned)p.extra ? 1 : 0);
+    const int ring = p.ring;
+
+    // nothing of X or Y is touched before grid_dependency_wait() returns (see above)
+    grid_launch_dependents();
+    if (tid == 0) {
+        for (int s = 0; s < kMaxRing; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], kMmaWarps);
+            mbar_init(&ready[s], 4);
+            mbar_init(&done[s], 1);
+        }
+        *stop = 0;
+        fence_barrier_init();
+    }
+    if (warp == 0) {
+        // all 512 columns of tensor memory: one CTA fills an SM
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(smem + 112)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if constexpr (kMinProduct)          // of the sixteen k of the offsets' product only four are used: the rest multiplies zeros
+        for (int i = tid; i < 8 * kMinRun / 16; i += kTcThreads)
+            *reinterpret_cast<uint4*>(smem + p.sx_off + kInvBytes + 16 * i) = make_uint4(0, 0, 0, 0);
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + 112);
+    volatile unsigned* gen_seen = reinterpret_cast<volatile unsigned*>(smem + 72);   // generation before this CTA arrived
+
+    if (warp >= kMmaWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kTcProducerRegs));
+        RunCursor cur;
+        cur.init(p, first, spc, count);
+        if (warp > kMmaWarps) {
+            // --------------------------------------------------------- issue (one thread for two warpgroups) ---
+            if (warp > kMmaWarps + 2) return;
+            const int wg0 = 2 * (warp - kMmaWarps - 1);
+            const uint32_t xs = smem_u32(smem + p.x_off) >> 4, base = tmem + kRegionCols * wg0;
+            // B descriptors: K-adjacent core matrices kKGroup (offsets: 256) bytes apart, N-adjacent ones 128, no swizzle
+            const uint64_t desc0 = ((uint64_t)(kKGroup >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
+            const uint64_t desc_min = ((uint64_t)(256 >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
+            const uint32_t term2 = kPlanes ? plane_bytes >> 4 : 128 >> 4;      // from a descriptor of term 1 to that of term 2
+            const uint32_t mins = smem_u32(smem + p.sx_off + kInvBytes) >> 4;
+            uint32_t k[2] = {0, 0};                      // times issued for each of the two
+            for (int n = 0; n < count;) {
+                const MmaItem& mat = p.item[cur.it];
+                const int rows_left = (int)mat.rows - (cur.rs - mat.rs_begin) * T::kStageRows;      // from the stage's first on
+                for (int e = cur.left, j = cur.j; e > 0; --e, ++j, ++n)
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        const int wg = wg0 + w, part = T::kF16 ? 0 : wg & 1, kh = T::kF16 ? wg : wg >> 1;
+                        if (rows_left <= 128 * part) continue;
+                        if (!mbar_try_wait(smem_u32(&ready[wg]), k[w] & 1u) && !*stop && !mbar_wait_bounded(&ready[wg], k[w] & 1u)) {
+                            atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
+                            *stop = 1;
+                        }
+                        __syncwarp();
+                        if (*stop) continue;             // nothing further is issued
+                        tc_after_sync();
+                        if (elect_one()) {
+                            const uint32_t b0 = xs + (uint32_t)(j * (kStageCols / 8) + kh * (T::kF16 ? 8 : 16)) * (kKGroup >> 4);
+                            const uint32_t a = base + kRegionCols * w, d = a + 64;
+#pragma unroll
+                            for (int i = 0; i < (T::kF16 ? 4 : 8); ++i) {
+                                const uint32_t b = b0 + 2 * i * (kKGroup >> 4);
+                                const uint32_t acc = d + kAccStep * (i >> 1);
+                                tc_mma(acc, a + 8 * i, desc0 | (uint64_t)b, kTcDesc, (i & 1) != 0);
+                                tc_mma(acc, a + 8 * i, desc0 | (uint64_t)(b + term2), kTcDesc, true);
+                            }
+                            if constexpr (kMinProduct) {
+                                const uint32_t b = mins + (uint32_t)(2 * j + kh) * (kMinRun >> 4);
+                                tc_mma(d + 4 * kAccStep, a + kMinsCol, desc_min | (uint64_t)b, kTcDesc, false);
+                                tc_mma(d + 4 * kAccStep, a + kMinsCol, desc_min | (uint64_t)(b + term2), kTcDesc, true);
+                            }
+                            tc_commit(smem_u32(&done[wg]));
+                        }
+                        __syncwarp();
+                        ++k[w];
+                    }
+                cur.next(p, spc, count - n);
+            }
+            if (*stop) {
+                // the compute warps have stopped waiting: products under way end before tensor memory is given back
+                for (int w = 0; w < 2; ++w)
+                    if (k[w] > 0 && !mbar_wait_bounded(&done[wg0 + w], (k[w] - 1) & 1u))
+                        atomicExch(p.fault, (int)FAULT_DRAIN_TIMEOUT);
+            }
+            asm volatile("bar.arrive 2, %0;" ::"n"(kMmaComputeThreads + 64) : "memory");
+            return;
+        }
+        // ------------------------------------------------------------- producer (one thread) ---
+        if (lane != 0) return;
+        if (!p.early_weights) grid_dependency_wait();
+        const uint64_t policy = l2_evict_first_policy();
+        int n = 0, slot = 0;
+        uint32_t parity = 1;                             // (the first pass over the ring waits for nothing)
+        while (n < count && !*stop) {
+            const int y = (cur.rs - p.item[cur.it].rs_begin) * T::kStageRows;
+            const CUtensorMap* map = &maps.m[cur.it];
+            int x = cur.c * spc + cur.j;
+            for (int e = cur.left; e > 0; --e, ++n, ++x) {
+                if constexpr (DROP) {
+                    if (n >= p.drop_stage) break;
+                }
+                if (!mbar_wait_bounded(&empty[slot], parity)) {      // the slot's previous use
+                    atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
+                    *stop = 1;
+                }
+                if (*stop) break;
+                mbar_expect_tx(&full[slot], kStageBytes);    // a box always delivers all its bytes (zeros past the end)
+                uint8_t* dst = smem + p.w_off + (size_t)slot * kStageBytes;
+                if constexpr (T::kF16) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) tensor_load_2d(dst + u * TcF16::kSliceBytes, map, (x * 4 + u) * 32, y, &full[slot], policy);
+                } else {
+                    tensor_load_2d(dst, map, x * T::kXWords, y, &full[slot], policy);
+                }
+                if (++slot == ring) slot = 0, parity ^= 1u;
+            }
+            if constexpr (DROP) {
+                if (n >= p.drop_stage) break;
+            }
+            cur.next(p, spc, count - n);
+        }
+        if (*stop) {
+            // the consumers have stopped waiting: make sure nothing is still landing in shared memory (stage m,
+            // the latest armed use of its slot, is the (m / ring)-th use)
+            for (int m = n - 1; m >= 0 && m >= n - ring; --m)
+                if (!mbar_wait_bounded(&full[m % ring], (uint32_t)(m / ring) & 1u))
+                    atomicExch(p.fault, (int)FAULT_DRAIN_TIMEOUT);
+        }
+        return;
+    }
+
+    // ------------------------------------------------------------------- compute warps ---
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kTcComputeRegs));
+    grid_dependency_wait();
+    if (p.self_clear) {
+        // this CTA's share of Y, then its arrival at the grid barrier; nobody adds into Y before the barrier
+        // has completed (checked before the first flush, by which time it normally has)
+        for (int it = 0; it < p.n_items; ++it) {
+            const int64_t n = (int64_t)p.batch * p.item[it].rows, quads = n / 4;
+            const int64_t q0 = quads * blockIdx.x / gridDim.x, q1 = quads * (blockIdx.x + 1) / gridDim.x;
+            float4* y4 = reinterpret_cast<float4*>(p.item[it].Y);
+            for (int64_t i = q0 + tid; i < q1; i += kMmaComputeThreads) y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (blockIdx.x == 0 && tid < (int)(n - 4 * quads)) p.item[it].Y[4 * quads + tid] = 0.f;
+        }
+        compute_barrier();
+        if (tid == 0) {
+            unsigned gen, prev;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(gen) : "l"(p.grid_bar + 1) : "memory");
+            *gen_seen = gen;
+            // release: the stores above (ordered before this thread by the barrier) become visible device-wide to
+            // whoever observes the new generation; acquire: the last CTA to arrive has seen everybody's
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(p.grid_bar) : "memory");
+            if (prev == gridDim.x - 1) {
+                asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p.grid_bar), "r"(0u) : "memory");
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.grid_bar + 1) : "memory");
+            }
+        }
+    }
+    bool cleared = !p.self_clear;       // may this warp add into Y yet?
+    const int wg = warp >> 2, quarter = warp & 3;
+    const int part = T::kF16 ? 0 : wg & 1, kh = T::kF16 ? wg : wg >> 1;            // which 128 rows, which columns
+    const int my_row = 128 * part + 32 * quarter + lane;                            // of a stage
+    const uint32_t ta = tmem + kRegionCols * wg + ((32u * quarter) << 16), td = ta + 64;
+    const uint32_t ready_bar = smem_u32(ready + wg), done_bar = smem_u32(done + wg);
+    const uint32_t xs = smem_u32(smem + p.x_off), sx_base = smem_u32(smem + p.sx_off);
+    const uint32_t full0 = smem_u32(full);
+    const uint32_t wrow = smem_u32(smem + p.w_off) +
+                          (T::kF16 ? (uint32_t)wg * TcF16::kSliceBytes + 128u * my_row : (uint32_t)my_row * T::kPiece);
+    if constexpr (kMinProduct) {
+        // the unused k of the offsets' A operand
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(ta + kMinsCol), "r"(0u) : "memory");
+    }
+
+    constexpr int kPairs = CB / 2;
+    f2 y[kPairs];
+#pragma unroll
+    for (int i = 0; i < kPairs; ++i) y[i] = 0;
+
+    // Of the products under way: the scales, and where their activations' scales (and sums) are.
+    bool pending = false;
+    uint32_t done_parity = 0;
+    float d[4], mn[4];                                   // mn[0]: the factor of the offsets' product, or the four offsets
+    uint32_t inv = 0;
+    // The run under way
+    RunCursor cur;
+    cur.init(p, first, spc, count);
+    int cur_c = -1;
+    const float* cur_x = nullptr;
+    float* out = nullptr;                                // this lane's element of column 0, null when its row is past the end
+    int64_t out_rows = 0;
+    bool live = false;
+    int j = 0, left = 0;
+    uint32_t slot_off = 0, full_bar = full0, parity = 0;
+
+    auto wait = [&](uint32_t bar, uint32_t ph) {
+        if (!mbar_try_wait(bar, ph) && !*stop && !mbar_wait_bounded(bar, ph)) {
+            if (lane == 0) {
+                atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
+                *stop = 1;
+            }
+        }
+        __syncwarp();
+    };
+    // One turn per stage, and one more that only finishes the last products.
+    for (int n = 0;; ++n) {
+        const bool change = left == 0;                   // another run begins, or the last one has ended
+        bool new_x = false;
+        bool live_next = live;
+        if (change) {
+            live_next = false;
+            if (n < count) {
+                const MmaItem& mat = p.item[cur.it];
+                live_next = (int)mat.rows - (cur.rs - mat.rs_begin) * T::kStageRows > 128 * part;     // the warpgroup has rows
+                new_x = cur.c != cur_c || mat.X != cur_x;
+            }
+        }
+        uint32_t a[32];
+        float dn[2], mnn[2];                             // scales and offsets of the first 64 columns' blocks
+        uint32_t mw[2];
+        auto decode = [&](auto g_tag, float* dd, float* mm, uint32_t& m) {
+            typename T::template Row<decltype(g_tag)::value> raw;
+            raw.load(wrow + slot_off);
+            raw.frag(a);
+            raw.scales(dd);
+            if constexpr (kMinProduct) m = raw.mins(), mm[0] = raw.min_factor();
+            else if constexpr (T::kHasMin) raw.offset(mm);
+        };
+        auto fetch = [&]() {
+            wait(full_bar, parity);
+            if constexpr (T::kF16) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint4 v = lds_v4(wrow + slot_off + (uint32_t)((i ^ (my_row & 7)) << 4));
+                    a[4 * i] = v.x, a[4 * i + 1] = v.y, a[4 * i + 2] = v.z, a[4 * i + 3] = v.w;
+                }
+            } else if (kh == 0) {
+                decode(std::integral_constant<int, 0>{}, dn, mnn, mw[0]);
+            } else {
+                decode(std::integral_constant<int, 2>{}, dn, mnn, mw[0]);
+            }
+        };
+        if (live_next && !new_x) fetch();
+        if (pending) {
+            wait(done_bar, done_parity);
+            done_parity ^= 1u;
+            pending = false;
+            tc_after_sync();
+            f2 yp[kPairs];
+            constexpr int kUnits = T::kF16 ? 2 : kMinProduct ? 5 : 4;
+            constexpr int kAtOnce = kPlanes ? 1 : kUnits;      // units read back together
+#pragma unroll
+            for (int u0 = 0; u0 < kUnits; u0 += kAtOnce) {
+                uint32_t r[kAtOnce * CB];
+#pragma unroll
+                for (int u = 0; u < kAtOnce; ++u) tmem_ld<CB>(td + kAccStep * (u0 + u), r + u * CB);
+                tmem_ld_wait(r);
+#pragma unroll
+                for (int v = 0; v < kAtOnce; ++v) {
+                    const int u = u0 + v;
+                    const float f = T::kF16 ? 1.f : u == 4 ? mn[0] : d[u & 3];
+#pragma unroll
+                    for (int i = 0; i < kPairs; ++i) {
+                        const f2 q = pack2u(r[v * CB + 2 * i], r[v * CB + 2 * i + 1]);
+                        if constexpr (T::kF16) yp[i] = q;
+                        else yp[i] = u == 0 ? mul2(pack2(f, f), q) : fma2(pack2(f, f), q, yp[i]);
+                    }
+                    if constexpr (T::kF16) add_scaled(inv + 64 * u, yp, y);
+                    if constexpr (T::kHasMin && !kMinProduct) {
+                        // the block's offset times the sum of its activations
+                        f2 off[kPairs];
+#pragma unroll
+                        for (int i = 0; i < kPairs; ++i) off[i] = pack2(mn[u], mn[u]);
+                        add_scaled(sx_base + kInvBytes + ((inv - sx_base) >> 6) * (4 * kSxBlockBytes) + u * kSxBlockBytes, off, y);
+                    }
+                }
+            }
+            if constexpr (!T::kF16) add_scaled(inv, yp, y);
+        }
+        if (change) {
+            if (n > 0) {
+                // the run's sums of this lane's row into Y
+                if (!cleared) {
+                    // the grid barrier: every CTA has cleared its share of Y once the generation has moved on
+                    if (lane == 0 && !*stop) {
+                        const unsigned gen0 = *gen_seen;       // written before the barriers of the first conversion
+                        unsigned gen = gen0;
+                        for (uint32_t i = 0; i < kGridPolls && gen == gen0; ++i)
+                            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(gen) : "l"(p.grid_bar + 1) : "memory");
+                        if (gen == gen0) {
+                            atomicExch(p.fault, (int)FAULT_GRID_BARRIER_TIMEOUT);
+                            *stop = 1;
+                        }
+                    }
+                    __syncwarp();
+                    cleared = true;
+                }
+                if (out) {
+                    float* o = out;
+#pragma unroll
+                    for (int i = 0; i < kPairs; ++i) {
+                        float v0, v1;
+                        unpack2(y[i], v0, v1);
+                        if (2 * i < p.batch) atomicAdd(o, v0);
+                        o += out_rows;
+                        if (2 * i + 1 < p.batch) atomicAdd(o, v1);
+                        o += out_rows;
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < kPairs; ++i) y[i] = 0;
+            }
+            if (n == count) break;
+            const MmaItem& mat = p.item[cur.it];
+            const int r = (cur.rs - mat.rs_begin) * T::kStageRows + my_row;
+            out_rows = mat.rows;
+            out = r < (int)out_rows ? mat.Y + r : nullptr;
+            live = live_next;
+            j = cur.j, left = cur.left;
+            if (new_x) {
+                cur_c = cur.c;
+                cur_x = mat.X;
+                tc_before_sync();
+                compute_barrier();                      // every warp is done with the previous chunk
+                // the chunk's activations as f16 terms, only the 256-column pieces this CTA's stages inside the chunk will read
+                const int64_t in_chunk = (int64_t)(mat.same_x_end - cur.rs) * spc - j;    // stages ahead that read this X
+                const int ahead = count - n;
+                const int m = (int)(in_chunk < ahead ? in_chunk : ahead), runs = 2 * (m < spc ? m : spc);
+                const float* src = mat.X + (int64_t)cur_c * Kx;
+                // a task is 128 columns (a run) of one activation column: a warp, four columns per lane.  Four loads in flight.
+                const int tasks = runs * p.batch;
+                const uint32_t recip = 65536u / (uint32_t)runs + 1u;          // task / runs, exactly (below 128)
+                for (int t0 = warp; t0 < tasks; t0 += 4 * kMmaWarps) {
+                    float4 v[4];
+                    int bs[4], k4s[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int task = t0 + q * kMmaWarps;
+                        const int b = (int)(((uint32_t)task * recip) >> 16), run = task - b * runs;
+                        int piece = j + (run >> 1);
+                        if (piece >= spc) piece -= spc;
+                        bs[q] = b;
+                        k4s[q] = piece * (kStageCols / 4) + 32 * (run & 1) + lane;
+                        if (task < tasks) v[q] = __ldg(reinterpret_cast<const float4*>(src + (int64_t)b * p.cols) + k4s[q]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (t0 + q * kMmaWarps >= tasks) break;
+                        const int b = bs[q], k4 = k4s[q];
+                        // f16: one scale per 32 columns (eight lanes), which brings the largest to 2^14..2^15; bf16: one per
+                        // 128, to 2^126..2^127, and 1 / s times 2^109 (2^24 of 2^133 is in the scales)
+                        constexpr int kLargest = T::kF16 ? 14 : 126, kUnit = T::kF16 ? 0 : 109, kLanes = T::kF16 ? 8 : 32;
+                        float mx = fmaxf(fmaxf(fabsf(v[q].x), fabsf(v[q].y)), fmaxf(fabsf(v[q].z), fabsf(v[q].w)));
+#pragma unroll
+                        for (int o = 1; o < kLanes; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                        int se = 254 + kLargest - (int)((__float_as_uint(mx) >> 23) & 0xFFu);      // biased exponent of s
+                        se = se > 253 ? 253 : se;
+                        // (bit 2 of lane: the upper 16 of a block of 32)
+                        const float sc0 = __uint_as_float((uint32_t)se << 23);
+                        const float sc = T::kUpperScaled && (lane & 4) ? sc0 * 0.0625f : sc0;
+                        if ((lane & (kLanes - 1)) == 0)
+                            *reinterpret_cast<float*>(smem + p.sx_off + (size_t)(k4 / kLanes) * 64 + 4 * b) =
+                                __uint_as_float((uint32_t)(254 + kUnit - se) << 23);
+                        if constexpr (T::kHasMin) {
+                            // sum of each block of 32 activations (eight consecutive lanes hold one)
+                            float sum = (v[q].x + v[q].y) + (v[q].z + v[q].w);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+                            if constexpr (kMinProduct) {
+                                // sum * s / 64 as three bf16 terms (exactly): [run][k / 8][n][k]; k = block of the run, term 1 in n
+                                // 0-7, term 2 in n 8-15, and term 3 in n 0-7 of k = 4 + block, where A repeats
+                                const float t = sum * (sc0 * 0.015625f);
+                                const float r1 = t - __uint_as_float(__float_as_uint(t) & 0xFFFF0000u);
+                                const float r2 = r1 - __uint_as_float(__float_as_uint(r1) & 0xFFFF0000u);
+                                const uint32_t h1 = __float_as_uint(t) >> 16, h2 = __float_as_uint(r1) >> 16, h3 = __float_as_uint(r2) >> 16;
+                                if ((lane & 7) == 0) {
+                                    uint8_t* at = smem + p.sx_off + kInvBytes + (size_t)(k4 >> 5) * kMinRun + 16 * b + 2 * (lane >> 3);
+                                    *reinterpret_cast<uint16_t*>(at) = (uint16_t)h1;
+                                    *reinterpret_cast<uint16_t*>(at + 128) = (uint16_t)h2;
+                                    *reinterpret_cast<uint16_t*>(at + 8) = (uint16_t)h3;
+                                }
+                            } else if ((lane & 7) == 0) {
+                                // [block of the chunk][column]
+                                *reinterpret_cast<float*>(smem + p.sx_off + kInvBytes + (size_t)(k4 >> 3) * kSxBlockBytes + 4 * b) = sum;
+                            }
+                        }
+                        const float x1 = T::kQuad ? v[q].z : v[q].y, x2 = T::kQuad ? v[q].y : v[q].z;
+                        uint32_t a0, a1, b0, b1;
+                        split_pair<T::kF16>(v[q].x * sc, x1 * sc, a0, b0);
+                        split_pair<T::kF16>(x2 * sc, v[q].w * sc, a1, b1);
+                        const uint32_t dst = xs + (uint32_t)(k4 >> 1) * kKGroup + 16u * b + 8u * (k4 & 1);
+                        const uint32_t dst2 = dst + (kPlanes ? plane_bytes : 128u);
+                        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst), "r"(a0), "r"(a1) : "memory");
+                        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst2), "r"(b0), "r"(b1) : "memory");
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the products read B through the async proxy
+                compute_barrier();
+                if (live) fetch();
+            }
+            cur.next(p, spc, count - n - left);
+        }
+        if (live) {
+            tmem_st32(ta, a);
+            if constexpr (!T::kF16) {
+                d[0] = dn[0], d[1] = dn[1];
+                float* mm = kMinProduct ? mn + 1 : mn + 2;
+                mn[0] = kMinProduct ? 64.f * mnn[0] : mnn[0];
+                if (!kMinProduct) mn[1] = mnn[1];
+                if (kh == 0) decode(std::integral_constant<int, 1>{}, d + 2, mm, mw[1]);
+                else decode(std::integral_constant<int, 3>{}, d + 2, mm, mw[1]);
+                tmem_st32(ta + 32, a);
+                if constexpr (kMinProduct)
+                    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %1, %2};" ::"r"(ta + kMinsCol), "r"(mw[0]), "r"(mw[1]) : "memory");
+            }
+            __syncwarp();                                // the stage's codes are out of shared memory
+            if (lane == 0) mbar_arrive(reinterpret_cast<uint64_t*>(smem + (full_bar - full0) + 8 * kMaxRing));
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_before_sync();
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ready_bar) : "memory");
+            pending = true;
+            inv = sx_base + (uint32_t)(T::kF16 ? 8 * j + 2 * wg : 2 * j + kh) * 64;
+        } else {
+            // (not before the stage has landed: an arrival ahead of that would count for an earlier use of the slot)
+            wait(full_bar, parity);
+            if (lane == 0) mbar_arrive(reinterpret_cast<uint64_t*>(smem + (full_bar - full0) + 8 * kMaxRing));
+        }
+        ++j, --left;
+        slot_off += kStageBytes, full_bar += 8;
+        if (full_bar == full0 + 8u * ring) slot_off = 0, full_bar = full0, parity ^= 1u;
+    }
+    // this CTA's share of the next launch's outputs (complete, like everything else here, when this grid completes)
+    for (int it = 0; it < p.n_next; ++it) {
+        const int64_t quads = p.next_n[it] / 4;
+        const int64_t q0 = quads * blockIdx.x / gridDim.x, q1 = quads * (blockIdx.x + 1) / gridDim.x;
+        float4* y4 = reinterpret_cast<float4*>(p.next_y[it]);
+        for (int64_t i = q0 + tid; i < q1; i += kMmaComputeThreads) y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (blockIdx.x == 0 && tid < (int)(p.next_n[it] - 4 * quads)) p.next_y[it][4 * quads + tid] = 0.f;
+    }
+    tc_before_sync();
+    asm volatile("bar.sync 2, %0;" ::"n"(kMmaComputeThreads + 64) : "memory");     // and the issuing warps are through
+    tc_after_sync();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
 template <class T, int NT, bool DROP = false>
@@ -1238,6 +1862,75 @@ int launch_mma(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_by
     return (int)cudaLaunchKernelEx(&cfg, matvec_mma_kernel<T, NT, DROP>, p, maps);
 }
 
+template <class T>
+int launch_mma_columns(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
+    return p.batch <= 8 ? launch_mma<T, 1>(p, maps, grid, smem_bytes, overlap, stream)
+                        : launch_mma<T, 2>(p, maps, grid, smem_bytes, overlap, stream);
+}
+
+template <class T, int CB, bool DROP = false>
+int launch_tc(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(matvec_tc_kernel<T, CB, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
+        if (e != cudaSuccess) return (int)e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    if (p.self_clear) {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = (p.self_clear || overlap) ? 1 : 0;
+    return (int)cudaLaunchKernelEx(&cfg, matvec_tc_kernel<T, CB, DROP>, p, maps);
+}
+
+// A launch holds 4, 8 or 16 columns (fewer accumulator columns to read back).
+template <class T>
+int launch_tc_columns(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
+    if (p.batch <= 4) return launch_tc<T, 4>(p, maps, grid, smem_bytes, overlap, stream);
+    if constexpr (T::kF16)
+        if (p.batch > 8) return launch_tc<T, 16>(p, maps, grid, smem_bytes, overlap, stream);
+    return launch_tc<T, 8>(p, maps, grid, smem_bytes, overlap, stream);
+}
+// Which launches take the tcgen05 kernel.  f16: all.  Quantised formats: up to eight columns of q4_K, q4_0, q8_0 and four of
+// q4_1, when there are enough stages (256 rows x 256 columns) per SM: a stage is cheaper there, but the first one takes
+// about 1 us longer to get through (conversion with scales, decode -> tensor memory -> product -> read back, nothing of it
+// overlapped yet).  Measured, us, warp-level -> tcgen05, 3 or 4 | 8 columns:
+//   q4_K  28672 x 4096 (12.1 stages per SM) 29.3 -> 21.9 | 29.2 -> 25.4   8192 x 4096 (3.5) 11.4 -> 10.6 | 11.5 -> 12.0
+//   q4_0  28672 x 4096                      25.3 -> 22.2 | 25.2 -> 24.3   8192 x 4096       10.0 -> 10.4 | 10.2 -> 11.4
+//   q8_0  28672 x 4096                      30.4 -> 26.8 | 30.4 -> 28.9   8192 x 4096       11.8 -> 11.5 | 12.1 -> 12.8
+//   q4_1  28672 x 4096                      26.7 -> 22.0 | 26.6 -> 27.4   (its offsets are applied in fp32)
+// q5_0, q5_1 and q5_K measured slower or equal (their fifth bits cost as much to place in either form); q6_K and q2_K have
+// scales per 16 weights and row pieces off the 16-byte grid; 9 to 16 columns spill (64 sums to read back per lane and stage).
+bool takes_tc(int fmt, int64_t n_stages, int batch) {
+    if (fmt == LW_F16) return true;
+    int per_sm;
+    switch (fmt) {
+        case LW_Q4_K: per_sm = 4; break;
+        case LW_Q4_0:
+        case LW_Q8_0: per_sm = batch <= 4 ? 4 : 7; break;
+        case LW_Q4_1:
+            if (batch > 4) return false;
+            per_sm = 4;
+            break;
+        default: return false;
+    }
+    return batch <= 8 && n_stages >= (int64_t)per_sm * device_sm_count();
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point lookup (no link against the driver library)
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1254,7 +1947,7 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-int mma_stage_rows(int fmt) { return fmt == LW_F16 ? MmaF16::kStageRows : kStageRows; }
+int mma_stage_rows(int fmt) { return fmt == LW_F16 ? TcF16::kStageRows : kStageRows; }
 
 // The weight matrix as a 2-D tensor of 32-bit words (row_bytes / 4 per row, `rows` rows) with boxes of one stage;
 // f16: boxes of one 128-byte slice of a stage's rows, written with the 128-byte swizzle.
@@ -1287,7 +1980,7 @@ unsigned* grid_barrier_words() {
 
 // Shared-memory plan of a launch: the largest chunk (1024, 512, 256 columns) that divides cols and leaves room
 // for at least two stages.  Returns false if nothing fits.
-bool mma_plan(int fmt, int64_t cols, int nt, int& chunk_cols, int& ring, size_t& x_bytes, size_t& stage_bytes,
+bool mma_plan(int fmt, bool tc, int64_t cols, int nt, int& chunk_cols, int& ring, size_t& x_bytes, size_t& stage_bytes,
               size_t& extra_bytes) {
     const int piece = fmt == LW_Q8_0   ? MmaQ80::kPiece
                       : fmt == LW_Q4_0 ? MmaQ40::kPiece
@@ -1298,15 +1991,29 @@ bool mma_plan(int fmt, int64_t cols, int nt, int& chunk_cols, int& ring, size_t&
                       : fmt == LW_Q5_1 ? MmaLegacy<LW_Q5_1>::kPiece
                       : fmt == LW_Q6_K ? MmaQ6K::kPiece
                       : fmt == LW_Q2_K ? MmaQ2K::kPiece
-                                       : MmaF16::kPiece;
+                                       : TcF16::kPiece;
     stage_bytes = (size_t)mma_stage_rows(fmt) * piece;
+    if (tc) {
+        // scales of the runs, then the sums of the blocks of 32: as B operand (4 KB) or as floats (2 KB)
+        extra_bytes = kInvBytes + 8 * kMinRun;
+        const size_t budget = kSmemPerCta - kMmaHeader - extra_bytes - 1024;      // (f16: up to 1 KB aligns the swizzled stages)
+        for (int kx = 1024; kx >= 256; kx /= 2) {
+            if (cols % kx != 0) continue;
+            x_bytes = (size_t)nt * (kx / 8) * kKGroup;
+            if (x_bytes + 2 * stage_bytes > budget) continue;
+            const size_t n = (budget - x_bytes) / stage_bytes;
+            ring = (int)(n > (size_t)kMaxRing ? kMaxRing : n);
+            chunk_cols = kx;
+            return true;
+        }
+        return false;
+    }
     // q4_K: block sums of the activations (64 bytes per block of a chunk of up to 1024 columns) and the warps' tables
     extra_bytes = fmt == LW_Q2_K ? (size_t)(1024 / 32) * 128 + (size_t)kMmaWarps * MmaQ2K::kTableBytes
                   : (fmt == LW_Q4_K || fmt == LW_Q5_K || fmt == LW_Q6_K)
                       ? (size_t)(1024 / 32) * kSxBlockBytes + (size_t)kMmaWarps * MmaQ4K::kTableBytes
-                      : ((fmt == LW_F16 || fmt == LW_Q4_1 || fmt == LW_Q5_1) ? (size_t)(1024 / 32) * kSxBlockBytes : 0);
-    // (f16: up to 1 KB more goes into aligning the swizzled stages)
-    const size_t budget = kSmemPerCta - kMmaHeader - extra_bytes - (fmt == LW_F16 ? 1024 : 0);
+                      : ((fmt == LW_Q4_1 || fmt == LW_Q5_1) ? (size_t)(1024 / 32) * kSxBlockBytes : 0);
+    const size_t budget = kSmemPerCta - kMmaHeader - extra_bytes;
     // the largest chunk that leaves room for two stages (q8_0, 458752 x 4096, 8 columns: 0.40 ms with chunks of
     // 1024 columns and two 68 KB stages against 0.49 ms with chunks of 256 and three)
     for (int kx = 1024; kx >= 256; kx /= 2) {
@@ -1359,6 +2066,10 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
     int* fault = device_fault_word();
     if (!fault) return (int)cudaErrorInvalidValue;
     if (pre_cleared) self_clear = false;
+    const int nt = batch > 8 ? 2 : 1;
+    int64_t n_stages = 0;
+    for (int i = 0; i < n_items; ++i) n_stages += (cols / kStageCols) * ((rows[i] + mma_stage_rows(fmt) - 1) / mma_stage_rows(fmt));
+    const bool tc = takes_tc(fmt, n_stages, batch);
     {
         // The grid barrier of the self-clearing form is one pair of words per device: it relies on two such
         // launches never running at the same time, which holds because each needs every SM to itself (cooperative
@@ -1366,7 +2077,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         // the clearing kernel instead.
         int cc = 0, rg = 0;
         size_t xb = 0, sb = 0, eb = 0;
-        if (!mma_plan(fmt, cols, batch > 8 ? 2 : 1, cc, rg, xb, sb, eb)) return (int)cudaErrorInvalidValue;
+        if (!mma_plan(fmt, tc, cols, nt, cc, rg, xb, sb, eb)) return (int)cudaErrorInvalidValue;
         if (2 * ((kMmaHeader + xb + eb + 127) / 128 * 128 + (size_t)rg * sb + 1024) <= 228 * 1024 || kCtasPerSm != 1)   // (f16's alignment slack only adds)
             self_clear = false;
     }
@@ -1397,10 +2108,9 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         const cudaError_t e = cudaLaunchKernelEx(&cfg, zero_kernel, z);
         if (e != cudaSuccess) return (int)e;
     }
-    const int nt = batch > 8 ? 2 : 1;
     MmaParams p{};
     size_t x_bytes = 0, stage_bytes = 0, extra_bytes = 0;
-    if (!mma_plan(fmt, cols, nt, p.chunk_cols, p.ring, x_bytes, stage_bytes, extra_bytes)) return (int)cudaErrorInvalidValue;
+    if (!mma_plan(fmt, tc, cols, nt, p.chunk_cols, p.ring, x_bytes, stage_bytes, extra_bytes)) return (int)cudaErrorInvalidValue;
     alignas(64) MmaMaps maps;
     const int64_t row_bytes = (int64_t)lw_row_bytes(fmt, cols);
     int rs = 0;
@@ -1432,9 +2142,11 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
     const size_t w_align = fmt == LW_F16 ? 1024 : 128;
     p.w_off = (uint32_t)((kMmaHeader + x_bytes + extra_bytes + w_align - 1) / w_align * w_align);
     const size_t smem_bytes = p.w_off + (size_t)p.ring * stage_bytes;
-    const int64_t n_stages = (cols / kStageCols) * (int64_t)rs;
     int grid = kCtasPerSm * device_sm_count();
     if ((int64_t)grid > n_stages && !self_clear) grid = (int)n_stages;   // self-clearing: every SM, so launches never overlap
+    p.share = (int)(n_stages / grid);
+    p.extra = (int)(n_stages % grid);
+    p.spc_shift = p.chunk_cols == 1024 ? 2 : p.chunk_cols == 512 ? 1 : 0;
     p.drop_stage = -1;
     p.n_next = n_next;
     for (int i = 0; i < n_next; ++i) {
@@ -1446,38 +2158,30 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         const int drop = take_drop_unit();
         if (drop >= 0) {
             p.drop_stage = drop;
-            return launch_mma<MmaQ40, 1, true>(p, maps, grid, smem_bytes, overlap != 0, stream);
+            return tc ? launch_tc<TcLegacy<LW_Q4_0>, 8, true>(p, maps, grid, smem_bytes, overlap != 0, stream)
+                      : launch_mma<MmaQ40, 1, true>(p, maps, grid, smem_bytes, overlap != 0, stream);
         }
     }
-    if (fmt == LW_Q4_0)
-        return nt == 1 ? launch_mma<MmaQ40, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaQ40, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q4_K)
-        return nt == 1 ? launch_mma<MmaQ4K, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaQ4K, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q5_K)
-        return nt == 1 ? launch_mma<MmaQ5K, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaQ5K, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_F16)
-        return nt == 1 ? launch_mma<MmaF16, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaF16, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q2_K)
-        return nt == 1 ? launch_mma<MmaQ2K, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaQ2K, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q6_K)
-        return nt == 1 ? launch_mma<MmaQ6K, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaQ6K, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q4_1)
-        return nt == 1 ? launch_mma<MmaLegacy<LW_Q4_1>, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaLegacy<LW_Q4_1>, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q5_0)
-        return nt == 1 ? launch_mma<MmaLegacy<LW_Q5_0>, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaLegacy<LW_Q5_0>, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    if (fmt == LW_Q5_1)
-        return nt == 1 ? launch_mma<MmaLegacy<LW_Q5_1>, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                       : launch_mma<MmaLegacy<LW_Q5_1>, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
-    return nt == 1 ? launch_mma<MmaQ80, 1>(p, maps, grid, smem_bytes, overlap != 0, stream)
-                   : launch_mma<MmaQ80, 2>(p, maps, grid, smem_bytes, overlap != 0, stream);
+    const bool ov = overlap != 0;
+    if (tc) switch (fmt) {
+        case LW_F16: return launch_tc_columns<TcF16>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q8_0: return launch_tc_columns<TcLegacy<LW_Q8_0>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_0: return launch_tc_columns<TcLegacy<LW_Q4_0>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_1: return launch_tc_columns<TcLegacy<LW_Q4_1>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_K: return launch_tc_columns<TcK4>(p, maps, grid, smem_bytes, ov, stream);
+    }
+    switch (fmt) {
+        case LW_Q8_0: return launch_mma_columns<MmaQ80>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_0: return launch_mma_columns<MmaQ40>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_1: return launch_mma_columns<MmaLegacy<LW_Q4_1>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q5_0: return launch_mma_columns<MmaLegacy<LW_Q5_0>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q5_1: return launch_mma_columns<MmaLegacy<LW_Q5_1>>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q4_K: return launch_mma_columns<MmaQ4K>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q5_K: return launch_mma_columns<MmaQ5K>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q2_K: return launch_mma_columns<MmaQ2K>(p, maps, grid, smem_bytes, ov, stream);
+        case LW_Q6_K: return launch_mma_columns<MmaQ6K>(p, maps, grid, smem_bytes, ov, stream);
+    }
+    return (int)cudaErrorInvalidValue;
 }
 
 int launch_matvec_mma(int fmt, const void* W, int64_t rows, int64_t cols, const float* X, float* Y, int batch,

@@ -398,3 +398,50 @@ def test_matvec_of_rows_off_the_16_byte_grid(fmt, rows, cols, overlap):
     check_matvec(y, y_ref, s_ref, "fmt %d %dx%d" % (fmt, rows, cols))
     X[0, cols // 2] = np.nan                       # every output reads it
     assert not np.isfinite(gpu_matvec(fmt, blocks, rows, cols, X, overlap=overlap)).any()
+
+
+# 256-column stages per SM decide between the two batched tensor-core kernels (4 and 7 times 148): sizes on the tcgen05
+# side, with a remainder of a warpgroup's 128 rows (1, 127, 129), chunks of 256, 512 and 1024 columns
+LARGE = [(lw.Q4_K, 30721, 1280, 3), (lw.Q4_K, 9599, 4096, 8), (lw.Q4_K, 75905, 512, 5), (lw.Q4_0, 30593, 1280, 4), (lw.Q4_0, 16513, 4096, 8),
+         (lw.Q4_0, 132735, 512, 5), (lw.Q4_1, 30721, 1280, 3), (lw.Q4_1, 9601, 4096, 4), (lw.Q8_0, 9599, 4096, 3), (lw.Q8_0, 53121, 1280, 8),
+         (lw.F16, 127, 256, 5), (lw.F16, 129, 1280, 9), (lw.F16, 1025, 2048, 16), (lw.F16, 257, 512, 3)]
+
+
+@pytest.mark.parametrize("fmt,rows,cols,batch", LARGE)
+def test_matvec_batched_large(fmt, rows, cols, batch):
+    # the tolerance is the contract's, in which a zero weight contributes exactly nothing: activations span 2^60 inside a run
+    # of 128 columns, wider than any fixed-point or f16 form could hold (q4_K, q4_1 and f16, whose statement is relative to
+    # the block's largest: ordinary activations)
+    n = min(rows, 3000)
+    some = quantized_weights(fmt, n, cols, seed=71, tensor_id=fmt, outlier_p=0.01).reshape(n, -1)
+    pick = np.random.default_rng(71).integers(0, n, rows)
+    pick[-n:] = np.arange(n)                         # the tail (checked against the oracle in full) has every row
+    blocks = np.ascontiguousarray(some[pick])
+    X = synth.activations(71, rows, batch, cols).reshape(batch, cols)
+    if fmt in (lw.Q4_0, lw.Q8_0):
+        X = np.ldexp(X, np.random.default_rng(72).integers(-50, 11, X.shape)).astype(np.float32)
+    y_ref, s_ref = oracle.matvec(fmt, some, n, cols, X, batch, nthreads=4)
+    y = gpu_matvec(fmt, blocks, rows, cols, X, batch, overlap=True, repeat=2).reshape(batch, rows)
+    check_matvec(y, np.asarray(y_ref).reshape(batch, n)[:, pick], np.asarray(s_ref).reshape(batch, n)[:, pick], "fmt %d" % fmt)
+
+
+def test_matvec_batched_large_group_and_copy_that_never_comes():
+    # two matrices that share X, one of its own, in one launch of the tcgen05 kernel; then the bounded wait of that kernel
+    rows, cols, batch = 4100, 4096, 3
+    ws = [quantized_weights(lw.Q4_0, rows, cols, seed=73, tensor_id=i) for i in range(3)]
+    xs = [synth.activations(73, i, batch, cols).reshape(batch, cols) for i in range(2)]
+    xd = [torch.from_numpy(x).cuda() for x in xs]
+    items = [(torch.from_numpy(w).cuda(), rows, xd[i > 1], torch.empty((batch, rows), device="cuda")) for i, w in enumerate(ws)]
+    lw.matvec_group(lw.Q4_0, cols, items, batch=batch)
+    torch.cuda.synchronize()
+    for i, w in enumerate(ws):
+        y_ref, s_ref = oracle.matvec(lw.Q4_0, w, rows, cols, xs[i > 1], batch, nthreads=4)
+        check_matvec(items[i][3].cpu().numpy(), np.asarray(y_ref), np.asarray(s_ref), "item %d" % i)
+    assert lw.device_status() == 0
+    lw.debug_drop_copy(1)
+    lw.matvec_group(lw.Q4_0, cols, items, batch=batch)
+    torch.cuda.synchronize()
+    assert lw.device_status() != 0
+    lw.matvec_group(lw.Q4_0, cols, items, batch=batch)
+    torch.cuda.synchronize()
+    assert lw.device_status() == 0
