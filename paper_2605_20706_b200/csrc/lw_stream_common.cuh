@@ -91,6 +91,9 @@ __device__ __forceinline__ void bulk_load_default(void* dst, const void* src, ui
         : "memory");
 }
 
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {      // both multiples of 16
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
