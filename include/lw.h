@@ -114,7 +114,7 @@ int lw_dequant(int fmt, const void* W_blocks, int64_t n, float* out, void* strea
  * Asynchronous on `stream`.
  * Accuracy.  With w the decoded weights and S = sum_k |w_k x_k|, every result satisfies
  *     |y - y_exact| <= 1e-4 * S + 1e-6 + E .
- * E = 0 for LW_VARIANT_GENERIC and for f16 at batch 1 and 2 (each weight is decoded exactly and then multiplied:
+ * E = 0 for LW_VARIANT_GENERIC when forced and for f16 at batch 1 and 2 (each weight is decoded exactly and then multiplied:
  * plain fp32 accumulation), for any finite input, and for the batched LW_VARIANT_TILE and LW_VARIANT_MMA on
  * q8_0, q4_0, q5_0 and q6_K (exact integer codes times the activations -- exact in TILE, to 2^-16 of each one's
  * own magnitude in MMA -- and block sums scaled in fp32) as long as |x| <= 2^115, which keeps a block's sum of
@@ -125,7 +125,8 @@ int lw_dequant(int fmt, const void* W_blocks, int64_t n, float* out, void* strea
  * that S does not cover.  For them
  *     E = c * sum_k What_k * A_k ,   c = 2^-18 (IDOT, the default for the quantised formats; MMA on q4_K, q5_K, q2_K,
  *                                    q4_1 and q5_1), 2^-16 (STREAM), 2^-30 (MMA on f16: activations as two f16
- *                                    terms relative to their block's largest),
+ *                                    terms relative to their block's largest; shapes that AUTO reports as GENERIC at
+ *                                    batch 1: 31-bit block fixed point, integer products, up to 16384 columns),
  * where, over the aligned run of 32 columns that contains k, A_k is the largest |x| and What_k the largest
  * decoded |w|.  This holds for weights made by lw_quantize, and for any block whose scale * code and offset
  * terms are at most four times its largest decoded magnitude.  The constants are worst-case figures (the
@@ -265,7 +266,8 @@ typedef enum {
                                with atomic additions (one per 1024 columns), so the last bits of a result can
                                differ from run to run.  Not chosen by AUTO (LW_VARIANT_MMA covers its shapes and
                                is faster); forced, it runs passes of 8 and 4 columns */
-    LW_VARIANT_MMA = 5      /* batch 2..16 only: tensor-core kernel (mma m16n8k16, bf16 operands, fp32 accumulation).
+    LW_VARIANT_MMA = 5      /* batch 2..16 only: tensor-core kernels (mma m16n8k16, and tcgen05.mma for f16 and for large
+                               launches of q4_K, q4_0, q4_1 and q8_0 with up to 8 columns; bf16 operands, fp32 accumulation).
                                A weight's integer code is exact in bf16 and the block scale is applied in fp32 to each
                                block's sum; every fp32 activation is cut into two bf16 terms that add up to it within
                                2^-16 of its magnitude (an error that scales with |w x| term by term and stays at
