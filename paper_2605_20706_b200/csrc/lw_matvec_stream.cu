@@ -70,8 +70,6 @@ namespace {
 
 // ------------------------------------------------------------------ kernel ---
 
-constexpr int64_t kPrefetchBytes = 32 * 1024;    // of a CTA's rows, sent to the L2 before the dependency wait
-
 struct StreamParams {
     const uint8_t* W;
     const float* X;
@@ -223,14 +221,18 @@ __global__ void __launch_bounds__(NG* kThreads, NG == 1 ? T::kMinCtas : 1)
     };
 
     LW_STAMP(1);
-    // While the previous kernel on the stream ends, HBM is idle: the first bytes of this CTA's rows go to the L2 (a hint, with
-    // no result: should that kernel still write W, the copies below read what it wrote).  The copies themselves, requested
-    // here, would keep the activations waiting behind them; an L2 prefetch does not use the way from the L2 to the SM.
-    // us per step without, 8, 16, 32, 48, 96 KB and everything: 1B q4_0 335, 321, 317, 317, 318, 323, 329; 8B q4_K
-    // 1273, 1258, 1251, 1247, 1248, 1253, 1314; 1B f16 from the host 593, 577, 569, 556, 557.
+    // While the previous kernel on the stream ends, HBM is idle: the first bytes of this CTA's rows go to the L2, behind its
+    // 512 bytes of the activations (a hint, with no result: should that kernel still write X or W, the loads below read what
+    // it wrote).  The copies themselves, requested here, would keep the activations waiting behind them; an L2 prefetch
+    // does not use the way from the L2 to the SM.  us per step without and with 8, 16, 32, 48, 96 KB of rows, activations
+    // already in the L2: 1B q4_0 335, 321, 317, 317, 318, 323; 8B q4_K 1273, 1258, 1251, 1247, 1248, 1253; 1B f16 562, 547,
+    // 540, 527.  Activations not in the L2, 8B q4_K in a graph: 1234; 1234 (16 KB), 1246 (32 KB) with the rows alone, 1211
+    // and 1216 with the activations in front.
     if (tid == 0 && rows_here > 0) {
+        constexpr int64_t most = T::kIntegerDot ? 16 * 1024 : 32 * 1024;
+        if (512 * (int64_t)cta < 4 * p.cols) l2_prefetch(Xm + 128 * cta, 512);       // (cols is a multiple of 256)
         const int64_t all = (int64_t)rows_here * row_bytes;
-        l2_prefetch(wbase, (uint32_t)(all < kPrefetchBytes ? all : kPrefetchBytes));
+        l2_prefetch(wbase, (uint32_t)(all < most ? all : most));
     }
     grid_dependency_wait();       // X may be produced, and Y still read, by the previous kernel
     LW_STAMP(2);
