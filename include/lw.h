@@ -114,8 +114,9 @@ int lw_dequant(int fmt, const void* W_blocks, int64_t n, float* out, void* strea
  * Asynchronous on `stream`.
  * Accuracy.  With w the decoded weights and S = sum_k |w_k x_k|, every result satisfies
  *     |y - y_exact| <= 1e-4 * S + 1e-6 + E .
- * E = 0 for LW_VARIANT_GENERIC when forced and for f16 at batch 1 and 2 (each weight is decoded exactly and then multiplied:
- * plain fp32 accumulation), for any finite input, and for the batched LW_VARIANT_TILE and LW_VARIANT_MMA on
+ * E = 0 for LW_VARIANT_GENERIC (forced, and where AUTO reports it) and for f16 at batch 1 and 2, for any finite input (each
+ * weight is decoded exactly and then multiplied, plain fp32 accumulation; the batch-1 integer kernel that serves most of
+ * these widths keeps every activation to 2^-14 of its own magnitude, ordinary ones to 2^-24), and for the batched LW_VARIANT_TILE and LW_VARIANT_MMA on
  * q8_0, q4_0, q5_0 and q6_K (exact integer codes times the activations -- exact in TILE, to 2^-16 of each one's
  * own magnitude in MMA -- and block sums scaled in fp32) as long as |x| <= 2^115, which keeps a block's sum of
  * code * x finite.  The streaming variants multiply the integer codes first and apply
@@ -125,8 +126,7 @@ int lw_dequant(int fmt, const void* W_blocks, int64_t n, float* out, void* strea
  * that S does not cover.  For them
  *     E = c * sum_k What_k * A_k ,   c = 2^-18 (IDOT, the default for the quantised formats; MMA on q4_K, q5_K, q2_K,
  *                                    q4_1 and q5_1), 2^-16 (STREAM), 2^-30 (MMA on f16: activations as two f16
- *                                    terms relative to their block's largest; shapes that AUTO reports as GENERIC at
- *                                    batch 1: 31-bit block fixed point, integer products, up to 16384 columns),
+ *                                    terms relative to their block's largest),
  * where, over the aligned run of 32 columns that contains k, A_k is the largest |x| and What_k the largest
  * decoded |w|.  This holds for weights made by lw_quantize, and for any block whose scale * code and offset
  * terms are at most four times its largest decoded magnitude.  The constants are worst-case figures (the
@@ -247,7 +247,9 @@ int lw_matvec_sequence_batch_host(int fmt, int n_items, const lw_seq_item* items
  * tunable work-group and tile sizes].  LW_VARIANT_AUTO lets the launch heuristics decide. */
 typedef enum {
     LW_VARIANT_AUTO = 0,
-    LW_VARIANT_GENERIC = 1, /* one warp per row, plain loads; any legal shape and batch */
+    LW_VARIANT_GENERIC = 1, /* one warp per row, plain loads; any legal shape and batch.  AUTO reports it for all widths
+                               that no streaming kernel takes; at batch 1 it runs an integer tensor-core kernel for
+                               most of them (same accuracy statement), at other batches this one */
     LW_VARIANT_STREAM = 2,  /* bulk-copy ring into shared memory, fp32 activations held in registers, one
                                512-thread CTA per SM; needs cols % 256 == 0, cols <= 16384 and rows that are
                                whole 16-byte pieces; batch 1.  Exists for f16, q8_0, q4_0 and q4_K; forced on

@@ -7,15 +7,21 @@
 // 32000 x 3072 63 -> 30 us, q4_0 11007 x 2848 18 -> 9.3 us (back to back from Python 10.6).
 //
 // Arithmetic.  The activations of a block of 32 (16 where the format's scales are per 16) become fixed point relative
-// to the block's largest: v = rint(x / d), |v| <= 2^30, d a power of two, so that every element down to 2^-7 of the
-// largest is represented exactly.  v is written as four signed digits of base 256.  mma.m16n8k32 (s8 x u8 / s8 -> s32)
+// to the block's largest M: v = rint(x / d), |v| < 2^31, d a power of two, so that every element down to 2^-6 M is
+// represented exactly and one of 2^-17 M to 2^-14 of itself.  What does not fit -- smaller elements beside a large one,
+// magnitudes of 2^96 and more, Inf and NaN -- counts as zero there and is multiplied in fp32 with its exactly decoded
+// weight: every element keeps a relative accuracy of its own, whatever stands beside it.  One element in 60 000 of normally
+// distributed activations is kept apart like this.
+// v is written as four signed digits of base 256.  mma.m16n8k32 (s8 x u8 / s8 -> s32)
 // multiplies A (16 x 32) = digits of the activations with B (32 x 8) = the codes of one block of 8 weight rows:
 //   A row m = g     : digit (g & 1)     of block s = g / 2 of the chain of four blocks,  g = 0..7
 //   A row m = g + 8 : digit 2 + (g & 1) of the same block
 // and zero in the rows of the other three blocks, so that four products accumulate into ONE set of accumulators
 // without mixing their blocks.  A lane then holds, for two rows, two digits of one block: it converts the exact integer
 // sums to fp32, multiplies them with d * 256^digit and with the block's weight scale, and adds them up.  An offset of
-// the code (q4_0's 8, q6_K's 32) is an integer too and goes into the accumulators' initial value, exactly.
+// the code (q4_0's 8, q6_K's 32) is an integer too and goes into the accumulators' initial value, exactly.  Where a block has
+// an offset of its own (q4_1, q5_1, q2_K), scale * sum of code * digit and offset * sum of digits nearly cancel when a large
+// activation meets a weight next to zero: they are added per digit, with one rounding.
 //
 // Work and data.  One CTA per SM: 16 compute warps and one copy warp.  The rows are cut evenly over the CTAs.  The copy warps bring tiles of rows into a ring of slots with 16-byte cp.async (rows
 // lie an odd multiple of 16 bytes apart in a slot, so the eight rows a warp reads at once fall into different banks;
@@ -30,6 +36,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "lw_internal.h"
 #include "lw_stream_common.cuh"
@@ -48,7 +55,10 @@ constexpr int kFoldRows = 128;                    // rows whose sums are collect
 constexpr int kTableFloats = kFoldRows * kComputeWarps;
 constexpr uint32_t kImmaHeader = 256;             // mbarriers, flags, zeros
 constexpr uint32_t kZeros = 160;                  // 96 bytes of zeros
-constexpr uint32_t kXBlock = 144;                 // bytes of a block of 32 activations: 4 digits x 32, scales and sums
+constexpr uint32_t kXBlock = 144;                 // bytes of a block of 32 activations: 4 digits x 32, scales
+constexpr uint32_t kApartBits = kImmaHeader + 2 * kTableFloats * 4;  // activations kept apart: one bit per column
+constexpr uint32_t kApartFrom = 0x6F800000u;      // 2^96: magnitudes from here on are kept apart
+constexpr uint32_t kApartBelow = 17u << 23;       // and those below 2^-17 of their unit's largest
 constexpr size_t kImmaSmemMax = 227 * 1024;
 
 struct ImmaParams {
@@ -75,6 +85,16 @@ struct ImmaParams {
 // ------------------------------------------------------------------ device helpers ---
 
 __device__ __forceinline__ void compute_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory"); }
+// the same, and whether any thread came with `v`
+__device__ __forceinline__ bool compute_bar_any(bool v) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)v), "n"(kComputeThreads)
+        : "memory");
+    return any != 0;
+}
 
 // 1-D bulk copy global -> shared, completion counted in bytes on `bar`; addresses and size are multiples of 16
 __device__ __forceinline__ void bulk_row(uint32_t dst, const uint8_t* src, uint32_t bytes, uint32_t bar, uint64_t policy) {
@@ -162,13 +182,24 @@ struct XState {
     float klo[CH], khi[CH];    // d * 256^digit of the lane's two digits (powers of two)
     float nlo[CH];             // -1.5 * 2^23 * klo
     int init[CH][4];           // initial accumulators: kIntMagic + code offset * sum of digits (digit lo twice, digit hi twice)
-    float sx[CH];              // sum of the unit's activations in the lanes with g even, else 0 (formats with an offset term)
+    float xlo[CH], xhi[CH];    // sums of the two digits (formats with an offset term)
 };
 
 // Integer sums (on top of kIntMagic: already the bit patterns of 1.5 * 2^23 + sum) of digits lo and hi of one unit and row
 // -> the unit's sum of code * x.  The scales are powers of two, so the first product is exact.
 __device__ __forceinline__ float unit_sum(int lo, int hi, float klo, float nlo, float khi) {
     return fmaf(__int_as_float(hi) - 12582912.f, khi, fmaf(__int_as_float(lo), klo, nlo));
+}
+// The same for a format with an offset term: the unit's sum of (d * code + m) * x onto acc.  Per digit d * S + m * X is
+// rounded once (and the error of m * X, where it can have one, is added back), so that a weight of zero takes its activation
+// out of the sum however large that is.  EXACT: m has 11 bits and X, a sum of 32 digits, 13.
+template <bool EXACT>
+__device__ __forceinline__ float affine_sum(int lo, int hi, float d, float m, float xlo, float xhi, float klo, float khi, float acc) {
+    const float sl = __int_as_float(lo) - 12582912.f, sh = __int_as_float(hi) - 12582912.f;
+    const float tl = __fmul_rn(m, xlo), th = __fmul_rn(m, xhi);
+    float rl = fmaf(d, sl, tl), rh = fmaf(d, sh, th);
+    if constexpr (!EXACT) rl = __fadd_rn(rl, fmaf(m, xlo, -tl)), rh = __fadd_rn(rh, fmaf(m, xhi, -th));
+    return fmaf(rh, khi, fmaf(rl, klo, acc));
 }
 struct RowPair {
     float a, b;                // sums of rows 2 t and 2 t + 1
@@ -225,6 +256,16 @@ struct ImmaLegacy {
     static constexpr bool kMayBeRagged = true;
     static constexpr bool kF16 = false;
 
+    static __device__ __forceinline__ float weight(uint32_t row, int c) {
+        const uint32_t b = row + (uint32_t)(c >> 5) * kBlock;
+        const float d = sh_half<0>(b);
+        if constexpr (kEight) return __fmul_rn((float)sh_s8<2>(b + (c & 31)), d);
+        const uint32_t nib = sh_u8<2 + (kHasMin ? 2 : 0) + (kFive ? 4 : 0)>(b + (c & 15));
+        int q = (int)(c & 16 ? nib >> 4 : nib & 15u);
+        if constexpr (kFive) q |= (int)((sh_u8<2 + (kHasMin ? 2 : 0)>(b + ((c & 31) >> 3)) >> (c & 7)) & 1u) << 4;
+        if constexpr (kHasMin) return __fadd_rn(__fmul_rn(d, (float)q), sh_half<2>(b));
+        return __fmul_rn((float)(q + kOffset), d);
+    }
     template <bool GEN, int J>
     static __device__ __forceinline__ void codes(const RowAddr& r, int t, uint32_t& b0, uint32_t& b1) {
         constexpr int B = J * kBlock;
@@ -266,13 +307,14 @@ struct ImmaLegacy {
                 const uint32_t s0 = R.s0[o] + s * kBlock, s1 = R.s1[o] + s * kBlock;
                 const float d0 = live ? sh_half<4 * CH * kBlock>(s0) : 0.f;
                 const float d1 = live ? sh_half<4 * CH * kBlock>(s1) : 0.f;
-                acc[o].a = fmaf(d0, unit_sum(c[o][0], c[o][2], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].a);
-                acc[o].b = fmaf(d1, unit_sum(c[o][1], c[o][3], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].b);
                 if constexpr (kHasMin) {
                     const float m0 = live ? sh_half<4 * CH * kBlock + 2>(s0) : 0.f;
                     const float m1 = live ? sh_half<4 * CH * kBlock + 2>(s1) : 0.f;
-                    acc[o].a = fmaf(m0, x.sx[CH], acc[o].a);
-                    acc[o].b = fmaf(m1, x.sx[CH], acc[o].b);
+                    acc[o].a = affine_sum<true>(c[o][0], c[o][2], d0, m0, x.xlo[CH], x.xhi[CH], x.klo[CH], x.khi[CH], acc[o].a);
+                    acc[o].b = affine_sum<true>(c[o][1], c[o][3], d1, m1, x.xlo[CH], x.xhi[CH], x.klo[CH], x.khi[CH], acc[o].b);
+                } else {
+                    acc[o].a = fmaf(d0, unit_sum(c[o][0], c[o][2], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].a);
+                    acc[o].b = fmaf(d1, unit_sum(c[o][1], c[o][3], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].b);
                 }
             }
         });
@@ -287,6 +329,12 @@ __device__ __forceinline__ float uint_float23(uint32_t v) { return __uint_as_flo
 struct ImmaQ6K {
     static constexpr bool kHasMin = false;
     static constexpr int kSuper = 210, kChains = 4, kGroup = 16, kOffset = -32;
+    static __device__ __forceinline__ float weight(uint32_t row, int c) {
+        const int h = c >> 7, j = (c >> 5) & 3, l = c & 31;
+        const uint32_t lo = sh_u8<0>(row + 64 * h + l + 32 * (j & 1)) >> (j & 2 ? 4 : 0), hi = sh_u8<128>(row + 32 * h + l) >> (2 * j);
+        const float dl = __fmul_rn(sh_half<208>(row), (float)sh_s8<192>(row + 8 * h + 2 * j + (l >> 4)));
+        return __fmul_rn(dl, (float)((int)((lo & 15u) | (hi & 3u) << 4) - 32));
+    }
     static constexpr bool kHalfScale = false, kMayStraddle = true, kMayBeRagged = true;
     static constexpr bool kF16 = false;
 
@@ -346,6 +394,12 @@ struct ImmaQ6K {
 struct ImmaQ2K {
     static constexpr bool kHasMin = true;
     static constexpr int kSuper = 84, kChains = 4, kGroup = 16, kOffset = 0;
+    static __device__ __forceinline__ float weight(uint32_t row, int c) {
+        const int h = c >> 7, j = (c >> 5) & 3, l = c & 31;
+        const uint32_t pair = sh_u8<0>(row + 8 * h + 2 * j + (l >> 4)), q = sh_u8<16>(row + 32 * h + l) >> (2 * j);
+        const float dl = __fmul_rn(sh_half<80>(row), (float)(pair & 15u)), ml = __fmul_rn(sh_half<82>(row), (float)(pair >> 4));
+        return __fsub_rn(__fmul_rn(dl, (float)(q & 3u)), ml);
+    }
     static constexpr bool kHalfScale = false, kMayStraddle = false, kMayBeRagged = true;
     static constexpr bool kF16 = false;
 
@@ -376,10 +430,8 @@ struct ImmaQ2K {
                     const uint32_t p0 = sh_u8<4 * CH>(R.s0[o] + s), p1 = sh_u8<4 * CH>(R.s1[o] + s);
                     const float e0 = d0[o] * (uint_float23(p0 & 15u) - 8388608.f), e1 = d1[o] * (uint_float23(p1 & 15u) - 8388608.f);
                     const float f0 = n0[o] * (uint_float23(p0 >> 4) - 8388608.f), f1 = n1[o] * (uint_float23(p1 >> 4) - 8388608.f);
-                    acc[o].a = fmaf(e0, unit_sum(c[0], c[2], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].a);
-                    acc[o].b = fmaf(e1, unit_sum(c[1], c[3], x.klo[CH], x.nlo[CH], x.khi[CH]), acc[o].b);
-                    acc[o].a = fmaf(f0, x.sx[CH], acc[o].a);
-                    acc[o].b = fmaf(f1, x.sx[CH], acc[o].b);
+                    acc[o].a = affine_sum<false>(c[0], c[2], e0, f0, x.xlo[CH], x.xhi[CH], x.klo[CH], x.khi[CH], acc[o].a);
+                    acc[o].b = affine_sum<false>(c[1], c[3], e1, f1, x.xlo[CH], x.xhi[CH], x.klo[CH], x.khi[CH], acc[o].b);
                 }
             });
         });
@@ -395,11 +447,12 @@ struct ImmaF16 {
 
 // ------------------------------------------------------------------ activations ---
 
-// X as fixed point in shared memory, blocks of 32 of kXBlock bytes: [digit 0..3][32 bytes] | {scale, sum} of the first
-// and of the second unit (one unit with GROUP 32).  A thread converts eight consecutive values; two (GROUP 16) or four
-// lanes share a unit.  X is read past L1: other SMs may have written it earlier in this launch.
-template <int GROUP, bool SUMS>
-__device__ __forceinline__ void convert_x(const float* X, int cols, int padded, uint32_t xs, int tid) {
+// X as fixed point in shared memory, blocks of 32 of kXBlock bytes: [digit 0..3][32 bytes] | scale of the first and of the
+// second unit (one unit with GROUP 32).  A thread converts eight consecutive values; two (GROUP 16) or four lanes share a
+// unit.  What does not fit a unit's fixed point gets its bit in `apart` (one per column); true if the thread met any.
+template <int GROUP>
+__device__ __forceinline__ bool convert_x(const float* X, int cols, int padded, uint32_t xs, uint8_t* apart, int tid) {
+    bool any = false;
     constexpr int kDepth = 2;                        // pieces of a thread whose loads are in flight together
     const int pieces = padded >> 3;                  // a multiple of 32: whole warps take part or drop out
     for (int p0 = tid; p0 < pieces; p0 += kDepth * kComputeThreads) {
@@ -417,24 +470,44 @@ __device__ __forceinline__ void convert_x(const float* X, int cols, int padded, 
         for (int j = 0; j < kDepth; ++j) {
             const int piece = p0 + j * kComputeThreads;
             if (piece >= pieces) break;
-            const float f[8] = {v[j][0].x, v[j][0].y, v[j][0].z, v[j][0].w, v[j][1].x, v[j][1].y, v[j][1].z, v[j][1].w};
-            uint32_t m = 0;
-            float sum = 0.f;
+            float f[8] = {v[j][0].x, v[j][0].y, v[j][0].z, v[j][0].w, v[j][1].x, v[j][1].y, v[j][1].z, v[j][1].w};
+            float most = 0.f, little = __uint_as_float(0x7F800000u);       // largest (NaN if any is) and smallest magnitude
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                m = max(m, __float_as_uint(f[i]) & 0x7FFFFFFFu);
-                sum += f[i];
+                asm("max.NaN.f32 %0, %0, %1;" : "+f"(most) : "f"(fabsf(f[i])));
+                little = fminf(little, fabsf(f[i]));
+            }
+            uint32_t m = __float_as_uint(most);
+            const bool far = __any_sync(0xFFFFFFFFu, m >= kApartFrom);
+            if (far) {
+                m = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t b = __float_as_uint(f[i]) & 0x7FFFFFFFu;
+                    m = max(m, b < kApartFrom ? b : 0u);
+                }
             }
             m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
             if (GROUP == 32) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-            if (SUMS) {
-                sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-                if (GROUP == 32) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+            // the scale 2^(e - 157) brings the unit's largest magnitude to 2^30 .. 2^31, below 0x7F7F7F80 (significands from
+            // 0xFEFEFF on take the next exponent): the top digit stays below 128
+            const uint32_t e = max((m + 0x10101u) >> 23, 31u);
+            const float up = __uint_as_float((284u - e) << 23);
+            const float d = __uint_as_float((e - 30u) << 23);
+            const uint32_t least = m > kApartBelow ? m - kApartBelow : 1u;
+            uint32_t bits = 0;
+            if (far || __float_as_uint(little) < least) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t b = __float_as_uint(f[i]) & 0x7FFFFFFFu;
+                    if (b - least >= kApartFrom - least) {         // below `least` or from kApartFrom on
+                        bits |= b != 0 ? 1u << i : 0u;
+                        f[i] = 0.f;
+                    }
+                }
             }
-            // the unit's largest magnitude lies in [2^(e - 127), 2^(e - 126)): the scale 2^(e - 156) brings it to 2^29 .. 2^30
-            const uint32_t e = max(m >> 23, 30u);
-            const float up = __uint_as_float((283u - e) << 23);
-            const float d = m >= 0x7F800000u ? __uint_as_float(0x7FC00000u) : __uint_as_float((e - 29u) << 23);
+            apart[piece] = (uint8_t)bits;
+            any |= bits != 0;
             uint32_t w[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) w[i] = ((uint32_t)__float2int_rn(f[i] * up) + 0x00808080u) ^ 0x00808080u;   // four signed digits
@@ -451,11 +524,37 @@ __device__ __forceinline__ void convert_x(const float* X, int cols, int padded, 
             for (int k = 0; k < 4; ++k)
                 asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst + 32u * k), "r"(dig[k][0]), "r"(dig[k][1]) : "memory");
             if ((piece & (GROUP / 8 - 1)) == 0)
-                asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(xs + (uint32_t)(piece >> 2) * kXBlock + 128u +
-                                                                     (GROUP == 16 ? 8u * ((piece >> 1) & 1) : 0u)),
-                             "f"(d), "f"(sum)
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(xs + (uint32_t)(piece >> 2) * kXBlock + 128u +
+                                                             (GROUP == 16 ? 4u * ((piece >> 1) & 1) : 0u)),
+                             "f"(d)
                              : "memory");
         }
+    }
+    return any;
+}
+
+// Adds weight * activation of the columns of a 256-column piece that are kept apart (bit table at `bits`, activations at X),
+// in fp32, to the row sums of a tile of n rows that the warp has just put into its table.  Eight rows at a time; the four
+// lanes of a row take the words of the bit table in turn.  `piece` = where the tile's row 0 has the piece in shared memory,
+// `at` = the table's entry of row 0, `shift0` = row 0's offset behind the boundary its copy started at, `rb` = what the next
+// row's offset differs by.
+template <class T>
+__device__ __noinline__ void add_apart(uint32_t piece, uint32_t pitch, uint32_t shift0, uint32_t rb, uint32_t at, uint32_t bits,
+                                       const float* X, int n, int first, int step, int lane) {
+    __syncwarp();
+    for (int u = first; u < n; u += step) {
+        const int i = u + (lane >> 2);
+        const uint32_t row = piece + (uint32_t)i * pitch + ((shift0 + (uint32_t)i * rb) & 15u);
+        float sum = 0.f;
+        for (int k = lane & 3; k < 8; k += 4)
+            for (uint32_t word = sh32(bits + 4u * k); word != 0; word &= word - 1) {
+                const int c = 32 * k + __ffs((int)word) - 1;
+                sum = fmaf(T::weight(row, c), X[c], sum);
+            }
+        __syncwarp();
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+        put_sum(at + (uint32_t)u * (4 * kComputeWarps) + 4u * (lane >> 2), sum, (lane & 3) == 0, true);
     }
 }
 
@@ -463,12 +562,13 @@ __device__ __forceinline__ void convert_x(const float* X, int cols, int padded, 
 template <class T>
 __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint32_t zeros, int g, int t) {
     const int s = g >> 1, odd = g & 1;
+    constexpr bool kSums = T::kOffset != 0 || T::kHasMin;
 #pragma unroll
     for (int ch = 0; ch < T::kChains; ++ch) {
         const int u = 4 * ch + s;
         const uint32_t blk = xb + (uint32_t)(T::kGroup == 32 ? u : u >> 1) * kXBlock;
         const uint32_t dig = blk + 32u * odd + 4u * t;
-        const uint32_t meta = blk + 128u + (T::kGroup == 32 ? 0u : 8u * (u & 1));
+        const uint32_t meta = blk + 128u + (T::kGroup == 32 ? 0u : 4u * (u & 1));
         int sum_lo, sum_hi;
         if constexpr (T::kGroup == 32) {
             // zeros are loaded, not selected: the compiler would redo 32 selections per group of rows to save registers
@@ -478,7 +578,7 @@ __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint3
                 const uint32_t from = s == j ? dig : zeros;
                 x.a[4 * ch + j][0] = sh32o<0>(from), x.a[4 * ch + j][1] = sh32o<64>(from);
                 x.a[4 * ch + j][2] = sh32o<16>(from), x.a[4 * ch + j][3] = sh32o<80>(from);
-                if constexpr (T::kOffset != 0) {
+                if constexpr (kSums) {
                     sum_lo = dp4a_ss(x.a[4 * ch + j][0], 0x01010101u, dp4a_ss(x.a[4 * ch + j][2], 0x01010101u, sum_lo));
                     sum_hi = dp4a_ss(x.a[4 * ch + j][1], 0x01010101u, dp4a_ss(x.a[4 * ch + j][3], 0x01010101u, sum_hi));
                 }
@@ -490,14 +590,14 @@ __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint3
                 const uint32_t from = s == 2 * q ? dig + 16u * (u & 1) : zeros, from2 = s == 2 * q + 1 ? dig + 16u * (u & 1) : zeros;
                 x.a[2 * ch + q][0] = sh32o<0>(from), x.a[2 * ch + q][1] = sh32o<64>(from);
                 x.a[2 * ch + q][2] = sh32o<0>(from2), x.a[2 * ch + q][3] = sh32o<64>(from2);
-                if constexpr (T::kOffset != 0) {
+                if constexpr (kSums) {
                     sum_lo = dp4a_ss(x.a[2 * ch + q][0], 0x01010101u, dp4a_ss(x.a[2 * ch + q][2], 0x01010101u, sum_lo));
                     sum_hi = dp4a_ss(x.a[2 * ch + q][1], 0x01010101u, dp4a_ss(x.a[2 * ch + q][3], 0x01010101u, sum_hi));
                 }
             }
         }
         x.init[ch][0] = x.init[ch][1] = x.init[ch][2] = x.init[ch][3] = kIntMagic;
-        if constexpr (T::kOffset != 0) {
+        if constexpr (kSums) {
             // the four lanes with equal g hold the unit's 32 (16) digits
             sum_lo += __shfl_xor_sync(0xFFFFFFFFu, sum_lo, 1), sum_hi += __shfl_xor_sync(0xFFFFFFFFu, sum_hi, 1);
             sum_lo += __shfl_xor_sync(0xFFFFFFFFu, sum_lo, 2), sum_hi += __shfl_xor_sync(0xFFFFFFFFu, sum_hi, 2);
@@ -509,7 +609,7 @@ __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint3
         x.klo[ch] = odd ? d * 256.f : d;
         x.khi[ch] = odd ? d * 16777216.f : d * 65536.f;
         x.nlo[ch] = -12582912.f * x.klo[ch];
-        x.sx[ch] = odd ? 0.f : __uint_as_float(sh32(meta + 4));
+        x.xlo[ch] = (float)sum_lo, x.xhi[ch] = (float)sum_hi;
     }
 }
 
@@ -519,7 +619,7 @@ template <class T>
 __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __grid_constant__ ImmaParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     // header: [0,64) full barriers | [64,128) empty barriers | 128 a wait gave up | [160,256) zeros
-    // then two tables of row sums, the activations, the ring of tiles
+    // then two tables of row sums, the bits of columns kept apart, the activations, the ring of tiles
     volatile int* gave_up = reinterpret_cast<volatile int*>(smem + 128);
     const uint32_t base = smem_u32(smem);
     const uint32_t full = base, empty = base + 64;
@@ -627,6 +727,7 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
     const uint32_t rb = p.row_bytes, pitch = p.pitch;
     const int rgrp = warp / chunk_sb, cw = warp - rgrp * chunk_sb;
     const bool ragged = p.ragged;
+    bool apart = false;                              // does any activation of the row not fit the fixed point?
     if constexpr (T::kF16) {
         for (int i = tid; i < nsb * 64; i += kComputeThreads) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -635,12 +736,13 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                          : "memory");
         }
     } else {
-        convert_x<T::kGroup, T::kHasMin>(p.X, p.cols, nsb * 256, xs, tid);
+        apart = convert_x<T::kGroup>(p.X, p.cols, nsb * 256, xs, smem + kApartBits, tid);
     }
-    compute_bar();
+    apart = compute_bar_any(apart);
     const uint32_t lane_g = (uint32_t)g * pitch + (uint32_t)cw * T::kSuper, lane_s = (uint32_t)(2 * t) * pitch + (uint32_t)cw * T::kSuper;
     const bool straddle = ragged || (((uint32_t)cw * T::kSuper) & 2u);
     XState<T::kChains> x;
+    bool piece_apart = false;                        // are there any in this warp's 256 columns?
     f2 xf[4];                                        // f16: the lane's eight activations
     for (int r0 = v0; r0 < v1; r0 += fold_rows) {
         const int r1 = min(v1, r0 + fold_rows);
@@ -657,6 +759,7 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                     xf[0] = pack2u(a.x, a.y), xf[1] = pack2u(a.z, a.w), xf[2] = pack2u(b.x, b.y), xf[3] = pack2u(b.z, b.w);
                 } else {
                     load_x<T>(x, xs + (uint32_t)(8 * sb) * kXBlock, base + kZeros, g, t);
+                    piece_apart = apart && __any_sync(0xFFFFFFFFu, sh32(base + kApartBits + 32u * sb + 4u * (lane & 7)) != 0);
                 }
             }
             const uint32_t coff = (uint32_t)c * chunk_sb * T::kSuper;
@@ -745,6 +848,9 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                         int u = 8 * rgrp;
                         for (; u + step < n; u += 2 * step) products(std::integral_constant<int, 2>{}, u);
                         if (u < n) products(std::integral_constant<int, 1>{}, u);
+                        if (piece_apart)
+                            add_apart<T>(tile + (uint32_t)cw * T::kSuper, pitch, ragged ? (uint32_t)r * rb + coff : 0u, ragged ? rb : 0u,
+                                         tab - 4u * (2 * t + (g & 1)), base + kApartBits + 32u * sb, p.X + 256 * sb, n, 8 * rgrp, step, lane);
                     }
                 }
                 __syncwarp();
@@ -800,7 +906,7 @@ bool plan(int fmt, int64_t rows, int64_t cols, int grid, ImmaParams& p, size_t& 
     p.chunk_sb = chunk_sb;
     p.n_chunks = chunks;
     p.row_groups = kComputeWarps / chunk_sb;
-    p.x_off = kImmaHeader + 2 * kTableFloats * 4;
+    p.x_off = kApartBits + 32u * nsb;
     p.ring_off = (uint32_t)((p.x_off + (size_t)nsb * (fmt == LW_F16 ? 1024 : 8 * kXBlock) + 127) & ~(size_t)127);
     const size_t margin = 1024;          // what a lane reads past the end of a row whose last piece is short lies inside
     const size_t avail = kImmaSmemMax - p.ring_off - margin;

@@ -304,3 +304,82 @@ def test_a_copy_that_never_comes_in_the_tensor_core_kernel(overlap):
         assert lw.device_status() == 0
     finally:
         lw.set_overlap(0)
+
+
+# widths that no streaming kernel takes: a batch-1 call there keeps the bound without an extra term, as for
+# LW_VARIANT_GENERIC (one row count below and two above the tile and CTA sizes of the kernel that runs them)
+OFF_GRID = [(lw.F16, 2848), (lw.Q8_0, 2848), (lw.Q4_0, 2848), (lw.Q4_1, 2848), (lw.Q5_0, 2848), (lw.Q5_1, 2848), (lw.Q6_K, 3072),
+            (lw.Q2_K, 2816), (lw.Q4_0, 8224), (lw.Q5_1, 8224), (lw.Q6_K, 8448), (lw.Q2_K, 8448)]
+
+
+@pytest.mark.parametrize("rows", [48, 700, 1481])
+@pytest.mark.parametrize("fmt,cols", OFF_GRID)
+def test_off_grid_widths_need_no_extra_term(fmt, cols, rows):
+    def check(blocks, X, what):
+        y_ref, s_ref = oracle.matvec(fmt, blocks, rows, cols, X, 1, nthreads=4)
+        y = _run(fmt, blocks, rows, cols, X)
+        finite = np.isfinite(y_ref.astype(np.float32)) & (s_ref < 3e38)
+        assert np.isfinite(y[finite]).all(), what
+        with np.errstate(invalid="ignore", over="ignore"):
+            ratio = np.abs(y.astype(np.float64) - y_ref) / (RTOL * s_ref + ATOL)
+        assert float(ratio[finite].max(initial=0.0)) <= 1.0, "%s: error / tolerance = %.3g" % (what, ratio[finite].max())
+
+    assert lw.query_variant(fmt, rows, cols, 1) == lw.VARIANT_GENERIC
+    rng = np.random.default_rng(300 + fmt)
+    for zero_rest in (False, True):
+        blocks, X = _adversarial(fmt, rows, cols, seed=90 + fmt, zero_rest_of_vector=zero_rest)
+        check(blocks, X, "outliers of 1e3..1e6 on zero weights")
+        hot = np.abs(X) >= 1e3
+        X[hot] = np.sign(X[hot]) * 64.0
+        check(blocks, X, "outliers of 64 on zero weights")
+    blocks = quantized_weights(fmt, rows, cols, seed=91, tensor_id=fmt)
+    X = np.ldexp(rng.standard_normal((1, cols)), rng.integers(-60, 20, (1, cols))).astype(np.float32)
+    check(blocks, X, "magnitudes over 2^80")
+    for value, where in ((1e30, 7), (2e38, cols - 1), (1e-41, 40), (2.0 ** -100, slice(None))):
+        X = np.zeros((1, cols), np.float32)
+        X[0, where] = value
+        check(blocks, X, "%g alone" % value)
+        X = X + synth.activations(92, fmt, 1, cols)
+        check(blocks, X.astype(np.float32), "%g beside ordinary activations" % value)
+    for bad, count in ((np.nan, 1), (np.inf, 1), (-np.inf, 2), (np.nan, 16), (np.inf, 40)):
+        X = synth.activations(93, fmt, 1, cols).copy()
+        X[0, cols - 64:cols - 64 + count] = bad
+        y = _run(fmt, blocks, rows, cols, X)
+        want = _run(fmt, blocks, rows, cols, X, lw.VARIANT_GENERIC)
+        assert not np.isfinite(y).any(), "%d of %r" % (count, bad)
+        np.testing.assert_array_equal(np.isnan(y), np.isnan(want))
+        np.testing.assert_array_equal(y[~np.isnan(y)], want[~np.isnan(want)])
+    lw.set_variant(lw.VARIANT_AUTO)
+    assert lw.device_status() == 0
+
+
+@pytest.mark.parametrize("large", [2.0 ** 10, 2.0 ** 15, 2.0 ** 24])
+@pytest.mark.parametrize("fmt", [lw.Q4_1, lw.Q5_1, lw.Q2_K])
+def test_off_grid_offsets_cancel_exactly(fmt, large):
+    # every row one block pattern with scale 1: a weight of exactly zero meets `large`, two others (-o and o + 1) meet 1,
+    # all else zero: the result is 1, whatever `large` is, and sum|w x| is small
+    if fmt == lw.Q2_K:
+        rows, cols, o = 700, 2816, 1
+        block = np.zeros(84, np.uint8)
+        block[:16] = 1 | (o << 4)                                     # weight = code - 1
+        block[80:84] = np.array([1.0, 1.0], np.float16).view(np.uint8)
+        codes = np.full(256, o)
+        codes[1], codes[2] = 0, o + 2                                 # -1, 2
+        for i, q in enumerate(codes):
+            block[16 + 32 * (i >> 7) + (i & 31)] |= q << (2 * ((i >> 5) & 3))
+    else:
+        rows, cols, o = 700, 2848, 7
+        codes = np.full(32, o)
+        codes[1], codes[2] = 0, 2 * o + 1                             # -7, 8
+        five = fmt == lw.Q5_1
+        block = np.zeros(24 if five else 20, np.uint8)
+        block[:4] = np.array([1.0, -float(o)], np.float16).view(np.uint8)
+        block[-16:] = codes[:16] | (codes[16:] << 4)
+    blocks = np.tile(block, rows * cols // len(codes))
+    X = np.zeros((1, cols), np.float32)
+    X[0, ::len(codes)] = np.random.default_rng(5).uniform(0.5, 1.0, cols // len(codes)) * large
+    X[0, 1::len(codes)] = X[0, 2::len(codes)] = 1.0
+    y_ref, s_ref = oracle.matvec(fmt, blocks, rows, cols, X, 1, nthreads=4)
+    y = _run(fmt, blocks, rows, cols, X)
+    worst = float((np.abs(y.astype(np.float64) - y_ref) / (RTOL * s_ref + ATOL)).max())
+    assert worst <= 1.0, "error / tolerance = %.3g" % worst
