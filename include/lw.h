@@ -91,8 +91,8 @@ const char* lw_status_string(int status);
  *         q = clamp(round(x/(d*scale)) + 32, 0, 63) (a deterministic rule of this library);
  *   f16 : round to nearest even.
  * src: host, n floats.  dst: host, lw_row_bytes(fmt, n) bytes, fully overwritten.  n must be a
- * whole number of blocks.  Pure CPU code: makes no CUDA call.  Single-threaded; callers may run
- * disjoint ranges from several threads. */
+ * whole number of blocks; a NaN or Inf among them fails the call and leaves dst as it was.  Pure CPU code: makes
+ * no CUDA call.  Single-threaded; callers may run disjoint ranges from several threads. */
 int lw_quantize(int fmt, const float* src, int64_t n, void* dst);
 
 /* Stand-alone dequantisation [Sec 3.3 decode routines]: out[i] = decode(W_blocks)[i] as fp32,

@@ -7,6 +7,8 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <memory>
+#include <new>
 #if defined(__x86_64__)
 #include <immintrin.h>
 #endif
@@ -738,12 +740,12 @@ static int rows_q6_K(const float* src, int64_t n, uint8_t* dst) {
     return LW_OK;
 }
 
-static int quantize(int fmt, const float* src, int64_t n, uint8_t* dst) {
+static int quantize_chunks(int fmt, const float* src, int64_t n, uint8_t* dst, bool check) {
     for (int64_t at = 0; at < n; at += kChunk) {
         const int64_t m = n - at < kChunk ? n - at : kChunk;
         const float* s = src + at;
         uint8_t* d = dst + lw_row_bytes(fmt, kChunk) * (size_t)(at / kChunk);
-        if (!all_finite(s, m)) return LW_ERR_NONFINITE;
+        if (check && !all_finite(s, m)) return LW_ERR_NONFINITE;
         int rc = LW_ERR_FORMAT;
         switch (fmt) {
             case LW_F16: rc = rows_f16(s, m, d); break;
@@ -760,6 +762,20 @@ static int quantize(int fmt, const float* src, int64_t n, uint8_t* dst) {
         if (rc != LW_OK) return rc;
     }
     return LW_OK;
+}
+
+// A non-finite weight anywhere leaves dst as it is.  The blocks go to a buffer and are copied when all of them are made, so that
+// main memory is read once (4 Mi weights: q4_K 3.6 -> 3.8 ms).  For f16, whose blocks are half as large as the weights, above
+// kHeldMost, or without the buffer, all weights are looked over first (q4_K 3.6 -> 4.6 ms).
+constexpr size_t kHeldMost = (size_t)32 << 20;
+static int quantize(int fmt, const float* src, int64_t n, uint8_t* dst) {
+    const size_t bytes = lw_row_bytes(fmt, n);
+    const bool hold = fmt != LW_F16 && bytes <= kHeldMost;
+    const std::unique_ptr<uint8_t[]> held(hold ? new (std::nothrow) uint8_t[bytes] : nullptr);
+    if (!held) return all_finite(src, n) ? quantize_chunks(fmt, src, n, dst, false) : LW_ERR_NONFINITE;
+    const int rc = quantize_chunks(fmt, src, n, held.get(), true);
+    if (rc == LW_OK) std::memcpy(dst, held.get(), bytes);
+    return rc;
 }
 
 static bool available() {

@@ -269,3 +269,17 @@ def test_quantiser_chunks_give_the_oracles_bytes(fmt, n):
     with pytest.raises(lw.LwError) as e:
         lw.quantize(fmt, x.reshape(-1))
     assert e.value.code == lw.ERR_NONFINITE
+
+
+@pytest.mark.parametrize("fmt", list(lw.FORMATS.values()))
+@pytest.mark.parametrize("n,at", [(256, 255), (4096 + 256, 4096), (64 * 4096, 64 * 4096 - 1), (64 * 4096, 32 * 4096 + 7)])
+def test_quantiser_that_refuses_writes_nothing(fmt, n, at):
+    # one non-finite weight, however late it comes: the call fails and the destination is as it was
+    x = np.random.default_rng(n + fmt).standard_normal(n, dtype=np.float32)
+    for bad in (np.nan, np.inf, -np.inf):
+        x[at] = bad
+        dst = np.full(lw.row_bytes(fmt, n), 0xA5, np.uint8)
+        with pytest.raises(lw.LwError) as e:
+            lw.quantize(fmt, x, dst)
+        assert e.value.code == lw.ERR_NONFINITE
+        assert (dst == 0xA5).all()
