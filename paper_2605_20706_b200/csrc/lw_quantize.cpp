@@ -100,7 +100,7 @@ static int quantize_rows_q4_0(const float* src, int64_t n, uint8_t* dst) {
         int arg = 0;
         for (int i = 1; i < 32; ++i)
             if (std::fabs(src[i]) > std::fabs(src[arg])) arg = i;   // first strict maximum of |x|
-        const float step = src[arg] / -8.f;
+        const float step = (src[arg] + 0.f) / -8.f;                 // (a block of zeros, of either sign: 0 / -8)
         const float inv = step != 0.f ? 1.f / step : 0.f;
         const uint16_t h = f32_to_f16_bits(step);
         if (is_inf_or_nan_half(h)) return LW_ERR_NONFINITE;
@@ -145,7 +145,7 @@ static int quantize_rows_legacy(const float* src, int64_t n, uint8_t* dst) {
             for (int i = 1; i < 32; ++i)
                 if (std::fabs(src[i]) > std::fabs(src[arg])) arg = i;   // first strict maximum of |x|
             constexpr float kHalf = (float)(1 << (BITS - 1));
-            const float step = src[arg] / -kHalf;
+            const float step = (src[arg] + 0.f) / -kHalf;               // (as in q4_0)
             const float inv = step != 0.f ? 1.f / step : 0.f;
             hd = f32_to_f16_bits(step);
             for (int i = 0; i < 32; ++i) {
@@ -498,7 +498,7 @@ static int rows_legacy(const float* src, int64_t n, uint8_t* dst) {
             __m256 y[4], m = _mm256_setzero_ps();
             for (int i = 0; i < 4; ++i) y[i] = abs8(x[i]), m = _mm256_max_ps(m, y[i]);
             constexpr float kHalf = (float)(1 << (BITS - 1));
-            step = src[first_equal(y, max_of(m))] / -kHalf;
+            step = (src[first_equal(y, max_of(m))] + 0.f) / -kHalf;
         }
         if (!plain_scale(step)) {
             const int rc = BITS == 4 && !OFFSET ? quantize_rows_q4_0(src, 32, dst) : quantize_rows_legacy<BITS, OFFSET>(src, 32, dst);

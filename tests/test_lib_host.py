@@ -283,3 +283,14 @@ def test_quantiser_that_refuses_writes_nothing(fmt, n, at):
             lw.quantize(fmt, x, dst)
         assert e.value.code == lw.ERR_NONFINITE
         assert (dst == 0xA5).all()
+
+
+@pytest.mark.parametrize("fmt", list(lw.FORMATS.values()))
+def test_quantiser_of_zeros_of_either_sign_and_subnormals_gives_the_oracles_bytes(fmt):
+    rng = np.random.default_rng(40 + fmt)
+    x = np.where(rng.random((64, 32)) < 0.5, np.float32(0.0), np.float32(-0.0)).astype(np.float32)
+    x[0], x[1] = 0.0, -0.0
+    np.testing.assert_array_equal(lw.quantize(fmt, x.reshape(-1)), oracle.quantize(fmt, x.reshape(-1)))
+    x[16:32] = rng.standard_normal((16, 32)) * 1e-38
+    x[32:48] = np.abs(rng.standard_normal((16, 32))) * 1e-41
+    np.testing.assert_array_equal(lw.quantize(fmt, x.reshape(-1)), oracle.quantize(fmt, x.reshape(-1)))
