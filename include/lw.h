@@ -402,8 +402,8 @@ int lw_probe_read(const void* src, int64_t bytes, void* stream);
  * records a fault, requests nothing further and returns; the rows of that unit and of the units after it are
  * left unwritten.  The batched tensor-core kernel has the same aid for q4_0 with up to 8 columns: the launch that
  * consumes the request asks for no copy from each CTA's u-th stage on, the wait for that stage runs out, the fault
- * is recorded and the kernel returns (its results are meaningless).  The request is consumed by the first launch of
- * either kind; u < 0 cancels it.  Always returns LW_OK. */
+ * is recorded and the kernel returns (its results are meaningless); so has the batch-1 integer kernel for q4_0, counted in
+ * tiles of rows.  The request is consumed by the first launch of any of these kinds; u < 0 cancels it.  Always returns LW_OK. */
 int lw_debug_drop_copy(int unit);
 
 #ifdef __cplusplus

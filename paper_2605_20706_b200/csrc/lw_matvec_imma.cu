@@ -79,6 +79,7 @@ struct ImmaParams {
     int chunk_sb;          // 256-column pieces of a row that are worked on at a time (<= 16, one per compute warp)
     int n_chunks;
     int row_groups;        // groups of compute warps that take different rows of a tile
+    int drop_tile;         // DROP builds only
     bool ragged;           // pieces do not start on 16-byte boundaries: every row's copy starts at the boundary below
 };
 
@@ -615,7 +616,8 @@ __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint3
 
 // ------------------------------------------------------------------ kernel ---
 
-template <class T>
+// DROP: testing aid, from tile p.drop_tile on nothing is requested (see lw_debug_drop_copy).
+template <class T, bool DROP = false>
 __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __grid_constant__ ImmaParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     // header: [0,64) full barriers | [64,128) empty barriers | 128 a wait gave up | [160,256) zeros
@@ -659,11 +661,17 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                 const uint32_t piece = min((uint32_t)p.chunk_sb * T::kSuper, rb - coff);
                 for (int r = r0; r < r1; r += tile_rows) {
                     const int n = min(tile_rows, r1 - r);
-                    if (*gave_up == 0 && !mbar_wait_bounded(empty + 8u * slot, parity)) {
+                    if constexpr (DROP) {
+                        if (issued >= p.drop_tile) return;       // (the compute warps still wait for what was requested)
+                    }
+                    // one decision for the warp: a compute warp may give up between two lanes' looks at the flag
+                    bool stop = *gave_up != 0;
+                    if (!stop && !mbar_wait_bounded(empty + 8u * slot, parity)) {
+                        stop = true;
                         *gave_up = 1;
                         atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
                     }
-                    if (*gave_up != 0) {
+                    if (__any_sync(0xFFFFFFFFu, stop)) {
                         // nothing further is requested; what is in flight lands before shared memory is released
                         for (int i = max(0, issued - slots); i < issued; ++i)
                             if (!mbar_wait_bounded(full + 8u * (i % slots), (uint32_t)(i / slots) & 1u))
@@ -924,14 +932,14 @@ bool plan(int fmt, int64_t rows, int64_t cols, int grid, ImmaParams& p, size_t& 
     return true;
 }
 
-template <class T>
+template <class T, bool DROP = false>
 int launch_one(const ImmaParams& p, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
     static bool attr_set[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(matvec_imma_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImmaSmemMax);
+        e = cudaFuncSetAttribute(matvec_imma_kernel<T, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImmaSmemMax);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
@@ -945,7 +953,7 @@ int launch_one(const ImmaParams& p, int grid, size_t smem_bytes, bool overlap, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, matvec_imma_kernel<T>, p);
+    return (int)cudaLaunchKernelEx(&cfg, matvec_imma_kernel<T, DROP>, p);
 }
 
 }  // namespace
@@ -966,6 +974,10 @@ int launch_matvec_imma(int fmt, const void* W, int64_t rows, int64_t cols, const
     p.W = static_cast<const uint8_t*>(W);
     p.X = X;
     p.Y = Y;
+    if (fmt == LW_Q4_0) {
+        p.drop_tile = take_drop_unit();
+        if (p.drop_tile >= 0) return launch_one<ImmaLegacy<LW_Q4_0>, true>(p, grid, smem, overlap, stream);
+    }
     switch (fmt) {
         case LW_F16: return launch_one<ImmaF16>(p, grid, smem, overlap, stream);
         case LW_Q8_0: return launch_one<ImmaLegacy<LW_Q8_0>>(p, grid, smem, overlap, stream);

@@ -383,3 +383,27 @@ def test_off_grid_offsets_cancel_exactly(fmt, large):
     y = _run(fmt, blocks, rows, cols, X)
     worst = float((np.abs(y.astype(np.float64) - y_ref) / (RTOL * s_ref + ATOL)).max())
     assert worst <= 1.0, "error / tolerance = %.3g" % worst
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+def test_a_copy_that_never_comes_in_the_integer_kernel(overlap):
+    # the same aid in the kernel for widths off the grid: from its second tile on a CTA requests nothing; the compute warps'
+    # wait runs out, the fault is recorded, the kernel ends, and the next call is an ordinary one
+    fmt, rows, cols = lw.Q4_0, 11007, 2848
+    blocks = quantized_weights(fmt, rows, cols, seed=99)
+    X = synth.activations(99, 0, 1, cols)
+    y_ref, s_ref = oracle.matvec(fmt, blocks, rows, cols, X, 1, nthreads=8)
+    assert lw.device_status() == 0
+    w = torch.from_numpy(blocks).cuda()
+    x = torch.from_numpy(X).cuda()
+    y = Guarded((1, rows))
+    lw.set_variant(lw.VARIANT_AUTO)
+    lw.set_overlap(overlap)
+    lw.debug_drop_copy(1)
+    lw.matvec(fmt, w, rows, cols, x, y.t, 1)
+    torch.cuda.synchronize()
+    y.check("Y of the faulted call")
+    assert lw.device_status() != 0
+    assert lw.device_status() == 0
+    check_matvec(_run(fmt, blocks, rows, cols, X), y_ref, s_ref, "call after the fault")
+    assert lw.device_status() == 0
