@@ -1431,12 +1431,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
                     for (int w = 0; w < 2; ++w) {
                         const int wg = wg0 + w, part = T::kF16 ? 0 : wg & 1, kh = T::kF16 ? wg : wg >> 1;
                         if (rows_left <= 128 * part) continue;
-                        if (!mbar_try_wait(smem_u32(&ready[wg]), k[w] & 1u) && !*stop && !mbar_wait_bounded(&ready[wg], k[w] & 1u)) {
-                            atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
-                            *stop = 1;
+                        // one decision for the warp: another warp may give up between two lanes' looks at the flag
+                        bool quit = false;
+                        if (!mbar_try_wait(smem_u32(&ready[wg]), k[w] & 1u)) {
+                            quit = *stop != 0;
+                            if (!quit && !mbar_wait_bounded(&ready[wg], k[w] & 1u)) {
+                                quit = true;
+                                atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
+                                *stop = 1;
+                            }
                         }
-                        __syncwarp();
-                        if (*stop) continue;             // nothing further is issued
+                        if (__any_sync(0xffffffffu, quit || *stop != 0)) continue;      // nothing further is issued
                         tc_after_sync();
                         if (elect_one()) {
                             const uint32_t b0 = xs + (uint32_t)(j * (kStageCols / 8) + kh * (T::kF16 ? 8 : 16)) * (kKGroup >> 4);
@@ -1460,11 +1465,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
                     }
                 cur.next(p, spc, count - n);
             }
-            if (*stop) {
+            if (__any_sync(0xffffffffu, *stop != 0)) {
                 // the compute warps have stopped waiting: products under way end before tensor memory is given back
                 for (int w = 0; w < 2; ++w)
                     if (k[w] > 0 && !mbar_wait_bounded(&done[wg0 + w], (k[w] - 1) & 1u))
                         atomicExch(p.fault, (int)FAULT_DRAIN_TIMEOUT);
+                __syncwarp();
             }
             asm volatile("bar.arrive 2, %0;" ::"n"(kMmaComputeThreads + 64) : "memory");
             return;
