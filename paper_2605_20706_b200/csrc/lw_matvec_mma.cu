@@ -1006,6 +1006,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             if constexpr (DROP) {
                 if (n >= p.drop_stage) break;
             }
+            if (n == ring && p.early_weights) grid_dependency_wait();    // (the previous kernel's time is not part of the bound)
             if (n >= ring && !mbar_wait_bounded(&empty[cur.slot], cur.parity ^ 1u)) {   // the slot's previous use
                 atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
                 *stop = 1;
@@ -1423,6 +1424,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
             const uint32_t term2 = kPlanes ? plane_bytes >> 4 : 128 >> 4;      // from a descriptor of term 1 to that of term 2
             const uint32_t mins = smem_u32(smem + p.sx_off + kInvBytes) >> 4;
             uint32_t k[2] = {0, 0};                      // times issued for each of the two
+            grid_dependency_wait();                      // (no A before that, and the previous kernel's time is not part of the bound)
             for (int n = 0; n < count;) {
                 const MmaItem& mat = p.item[cur.it];
                 const int rows_left = (int)mat.rows - (cur.rs - mat.rs_begin) * T::kStageRows;      // from the stage's first on
@@ -1489,6 +1491,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
                 if constexpr (DROP) {
                     if (n >= p.drop_stage) break;
                 }
+                if (n == ring && p.early_weights) grid_dependency_wait();    // (the previous kernel's time is not part of the bound)
                 if (!mbar_wait_bounded(&empty[slot], parity)) {      // the slot's previous use
                     atomicExch(p.fault, (int)FAULT_BULK_WAIT_TIMEOUT);
                     *stop = 1;
