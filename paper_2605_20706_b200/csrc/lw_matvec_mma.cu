@@ -18,9 +18,9 @@
 // (q4_0, q8_0; q4_K's sub-block offsets go onto fp32 sums of the activations and bring an extra term back, see MmaQ4K).
 //
 // Two kernels.  matvec_mma_kernel (mma.sync, described here) takes the fragments straight from the decode; it has every
-// quantised format and up to 16 columns.  matvec_tc_kernel (tcgen05.mma, further down) takes f16 and, up to eight columns,
-// large launches of q4_K, q4_0, q4_1 and q8_0 (takes_tc has the rule and the times): there a masked word of codes is an
-// operand of the product as it is, which is worth the extra store of every weight to tensor memory.
+// format and up to 16 columns.  matvec_tc_kernel (tcgen05.mma, further down) takes f16 but for small launches and, up to
+// eight columns, large launches of q4_K, q4_0, q4_1 and q8_0 (takes_tc has the rule and the times): there a masked word of
+// codes is an operand of the product as it is, which is worth the extra store of every weight to tensor memory.
 //
 // Layout of the work.  A stage is 256 rows x 256 columns of weights (36 KB of q4_0, 68 KB of q8_0), brought in
 // by a producer thread with one tiled bulk-tensor copy (the matrix as a 2-D tensor of 32-bit words; rows beyond
@@ -202,6 +202,7 @@ __device__ __forceinline__ uint32_t bytes_to_bf16_128_plus(uint32_t v) {
 // the row's piece of the stage plus 4 t (t = lane % 4), OFF = byte offset of the two-block unit from there.
 struct MmaQ40 {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 8 * 18;               // bytes of a row's 256 columns
@@ -234,6 +235,7 @@ struct MmaQ40 {
 
 struct MmaQ80 {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 8 * 34;
@@ -277,6 +279,7 @@ struct MmaQ80 {
 // accuracy statement).  The 6-bit fields are unpacked once per warp and stage into a table of (d * sc, dmin * m).
 struct MmaQ4K {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 144;
@@ -333,6 +336,7 @@ struct MmaQ4K {
 // s of byte l is the high bit of weight l of sub-block s, so a code is 0..31 -- still exact in bf16.
 struct MmaQ5K {
     static constexpr int kStageRows = 256;          // 16 warps x 16 rows
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     static constexpr int kPiece = 176;
@@ -397,6 +401,7 @@ struct MmaLegacy {
     static constexpr bool kHasMin = FMT != LW_Q5_0;
     static constexpr int kBlock = FMT == LW_Q4_1 ? 20 : (FMT == LW_Q5_0 ? 22 : 24);
     static constexpr int kStageRows = 256;
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = false;
     // 16 bytes more than a row's 256 columns are fetched for q4_1 and q5_1: their 160- and 192-byte pitches would put
@@ -444,6 +449,79 @@ struct MmaLegacy {
     }
 };
 
+// f16 weights: they are the A operand as they lie in memory (mma with f16 operands), nothing is decoded.  A row's
+// 256 columns are 512 bytes, fetched as four 128-byte slices (one per 64-column unit) with the 128-byte swizzle of
+// the tensor copy, so that the eight rows a warp reads at once fall into different banks: 16-byte chunk c of row r
+// of a slice sits at chunk c ^ (r % 8).  A stage is 128 rows; warps 0-7 take units 0 and 1 of their 16 rows, warps
+// 8-15 units 2 and 3.  The activations are held as f16 terms of x * s, s a power of two per block of 32 and
+// column that brings the block's largest magnitude to 2^14..2^15: the first term is cut off exactly, the second
+// rounds what is left (22 significant bits of the element, but nothing below 2^-38 of the block's largest
+// magnitude: the extra term E of the accuracy statement with a tiny constant); 1 / s multiplies the block's sum.
+struct MmaF16 {
+    static constexpr int kStageRows = 128;
+    static constexpr bool kF16 = true;
+    static constexpr bool kQ6K = false;
+    static constexpr bool kQ2K = false;
+    static constexpr int kPiece = 512;
+    static constexpr bool kHasMin = false;
+    static constexpr int kTableBytes = 0;
+    static constexpr int kSliceBytes = kStageRows * 128;     // one unit of all the stage's rows
+};
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                              uint32_t b0, uint32_t b1) {
+    asm("{\n\t.reg .f32 z;\n\tmov.f32 z, 0f00000000;\n\t"
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{z, z, z, z};\n\t}"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// One block of 32 f16 weights of the warp's 16 rows against all columns.  wrow = address of row g's 128 bytes in
+// slice 0 of the stage plus 8 (t % 2); sw[h] = byte offset of the lane's swizzled 16-byte chunk for half h of block
+// 0 (block 1: sw[2 + h]); sx = the lane's two block scales (1 / s), group nt 32 bytes further.
+template <int NT, int U, int BLK>
+__device__ __forceinline__ void block_step_f16(uint32_t wrow, const uint32_t (&sw)[4], uint32_t sx,
+                                               const uint32_t (&xp)[NT][kTerms], float (&y)[NT][4]) {
+    constexpr int kSlice = U * MmaF16::kSliceBytes;
+    uint32_t a[4], b[4];
+    lds64<kSlice>(wrow + sw[2 * BLK], a[0], a[1]);               // row g: k = 4t .. 4t+3
+    lds64<kSlice>(wrow + sw[2 * BLK + 1], a[2], a[3]);           //        k = 16+4t ..
+    lds64<kSlice + 8 * 128>(wrow + sw[2 * BLK], b[0], b[1]);     // row g + 8 (same swizzle: (g + 8) % 8 == g)
+    lds64<kSlice + 8 * 128>(wrow + sw[2 * BLK + 1], b[2], b[3]);
+    constexpr int kX = 2 * (64 * U + 32 * BLK);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        float c[4];
+#pragma unroll
+        for (int s = 0; s < kTerms; ++s) {
+            uint32_t b0, b1, b2, b3;
+            lds128<kX>(xp[nt][s], b0, b1, b2, b3);
+            if (s == 0)
+                mma_f16_first(c, a[0], b[0], a[1], b[1], b0, b1);
+            else
+                mma_f16(c, a[0], b[0], a[1], b[1], b0, b1);
+            mma_f16(c, a[2], b[2], a[3], b[3], b2, b3);
+        }
+        float s0, s1;                                            // 1 / s of columns 2 t and 2 t + 1 of the group
+        if (nt == 0)
+            lds_f32x2<kSxBlockBytes * (2 * U + BLK)>(sx, s0, s1);
+        else
+            lds_f32x2<kSxBlockBytes * (2 * U + BLK) + 32>(sx, s0, s1);
+        y[nt][0] = fmaf(s0, c[0], y[nt][0]);
+        y[nt][1] = fmaf(s1, c[1], y[nt][1]);
+        y[nt][2] = fmaf(s0, c[2], y[nt][2]);
+        y[nt][3] = fmaf(s1, c[3], y[nt][3]);
+    }
+}
+
 // q6_K: 210-byte super-blocks {128 bytes of low nibbles, 64 bytes of upper bit pairs, 16 int8 scales (one per 16
 // weights), d}.  210 is not a multiple of 16, so a row's piece of a stage starts anywhere on a 2-byte grid: the
 // tensor copy starts at the 16-byte boundary below it and fetches 240 bytes per row, and the kernel indexes from
@@ -454,6 +532,7 @@ struct MmaLegacy {
 // bytes l and l + 32) for even U and {2, 3} (high nibbles) for odd U.
 struct MmaQ6K {
     static constexpr int kStageRows = 256;
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = true;
     static constexpr bool kQ2K = false;
     static constexpr int kSuper = 210;                  // bytes of 256 weights
@@ -482,6 +561,7 @@ struct MmaQ6K {
 // sums of each 16 activations (extra term E, c = 2^-18).  Unit U = half U / 2, groups {0, 1} or {2, 3}.
 struct MmaQ2K {
     static constexpr int kStageRows = 256;
+    static constexpr bool kF16 = false;
     static constexpr bool kQ6K = false;
     static constexpr bool kQ2K = true;
     static constexpr int kSuper = 84;
@@ -713,6 +793,19 @@ __device__ __forceinline__ void split3(float x, uint32_t& h1, uint32_t& h2, uint
         h2 = b2 >> 16;
         h3 = __float_as_uint(r2) >> 16;                 // at most eight significant bits are left: exact
     }
+}
+
+// fp32 -> f16 terms of x (already scaled into the f16 range): cut off (exact differences) except the last, which
+// rounds the rest
+__device__ __forceinline__ void split3_f16(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
+    unsigned short a, b, c;
+    asm("cvt.rz.f16.f32 %0, %1;" : "=h"(a) : "f"(x));
+    const float r1 = x - __half2float(__ushort_as_half(a));
+    if (kTerms == 2) asm("cvt.rn.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
+    else asm("cvt.rz.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
+    const float r2 = r1 - __half2float(__ushort_as_half(b));
+    asm("cvt.rn.f16.f32 %0, %1;" : "=h"(c) : "f"(r2));
+    h1 = a, h2 = b, h3 = c;
 }
 
 // ------------------------------------------------------------------ tcgen05 kernel ---
@@ -1013,7 +1106,14 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                 break;
             }
             mbar_expect_tx(&full[cur.slot], kStageBytes);   // a box always delivers all its bytes (zeros past the end)
-            if constexpr (T::kQ6K || T::kQ2K) {
+            if constexpr (T::kF16) {
+                // four swizzled 128-byte slices (one per 64-column unit), each all the stage's rows
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    tensor_load_2d(smem + p.w_off + (size_t)cur.slot * kStageBytes + u * MmaF16::kSliceBytes,
+                                   &maps.m[cur.it], ((cur.c * spc + cur.j) * 4 + u) * 32,
+                                   (cur.rs - p.item[cur.it].rs_begin) * kStageRows, &full[cur.slot], policy);
+            } else if constexpr (T::kQ6K || T::kQ2K) {
                 // the piece starts at byte kSuper * (stage's column index) of the row: fetch from the 16-byte boundary below
                 tensor_load_2d(smem + p.w_off + (size_t)cur.slot * kStageBytes, &maps.m[cur.it],
                                ((T::kSuper * (cur.c * spc + cur.j)) >> 4) << 2,
@@ -1065,7 +1165,13 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
     const uint32_t xs = smem_u32(smem + p.x_off);
     // this lane's B fragments: column g of each group of eight, slots 8 t .. 8 t + 7 of a block of 32
     const uint32_t xlane = xs + g * x_pitch + 16u * t;
-    const uint32_t wrow = smem_u32(smem + p.w_off) + (uint32_t)(16 * warp + g) * kPiece;      // the warp's 16 rows of a stage
+    // the warp's 16 rows of a stage; f16: 128-row stages, warps 0-7 take units 0 and 1, warps 8-15 units 2 and 3
+    const int mt = T::kF16 ? (warp & 7) : warp;
+    const uint32_t wrow = smem_u32(smem + p.w_off) +
+                          (T::kF16 ? (uint32_t)(16 * mt + g) * 128u + 8u * (t & 1) : (uint32_t)(16 * warp + g) * kPiece);
+    uint32_t sw[4];                                     // f16: the lane's swizzled chunk offsets (see block_step_f16)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sw[i] = (uint32_t)(((2 * i + (t >> 1)) ^ g) << 4);
 
     float y[NT][4];
 #pragma unroll
@@ -1094,7 +1200,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             cleared = true;
         }
         const MmaItem& m = p.item[cur_it];
-        const int64_t r = (int64_t)(cur_rs - m.rs_begin) * kStageRows + 16 * warp + g;
+        const int64_t r = (int64_t)(cur_rs - m.rs_begin) * kStageRows + 16 * mt + g;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -1118,7 +1224,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             cur_it = cur.it;
         }
         if (c != cur_c || mat.X != cur_x) {
-            // the chunk's activations as one bf16 plane per term: plane s, column b.  Inside a block of 32 the order is
+            // the chunk's activations as one bf16 (f16) plane per term: plane s, column b.  Inside a block of 32 the order is
             // the one the fragments want: slots 8 q .. 8 q + 3 hold k = 4 q .. 4 q + 3 and slots 8 q + 4 .. 8 q + 7
             // hold k = 16 + 4 q .., so a lane reads both halves of its B operand with one 16-byte load.
             cur_c = c;
@@ -1152,10 +1258,29 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                         const int idx = tid + nt * kMmaComputeThreads;
                         const int b = idx >> 6, k4 = jj * (kStageCols / 4) + (idx & 63);
                         uint32_t h[3][4];
-                        split3(v[q][nt].x, h[0][0], h[1][0], h[2][0]);
-                        split3(v[q][nt].y, h[0][1], h[1][1], h[2][1]);
-                        split3(v[q][nt].z, h[0][2], h[1][2], h[2][2]);
-                        split3(v[q][nt].w, h[0][3], h[1][3], h[2][3]);
+                        if constexpr (T::kF16) {
+                            // f16 terms of x * s, s = the power of two that brings the block's largest magnitude (eight
+                            // consecutive lanes hold a block of 32) to 2^14 .. 2^15; 1 / s goes to [block][column]
+                            float mx = fmaxf(fmaxf(fabsf(v[q][nt].x), fabsf(v[q][nt].y)), fmaxf(fabsf(v[q][nt].z), fabsf(v[q][nt].w)));
+                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                            int se = 268 - (int)((__float_as_uint(mx) >> 23) & 0xFFu);      // biased exponent of s
+                            se = se < 1 ? 1 : (se > 253 ? 253 : se);
+                            const float sc = __uint_as_float((uint32_t)se << 23);
+                            if ((lane & 7) == 0)
+                                *reinterpret_cast<float*>(smem + p.sx_off + (size_t)(k4 >> 3) * kSxBlockBytes + 4 * b) =
+                                    __uint_as_float((uint32_t)(254 - se) << 23);
+                            split3_f16(v[q][nt].x * sc, h[0][0], h[1][0], h[2][0]);
+                            split3_f16(v[q][nt].y * sc, h[0][1], h[1][1], h[2][1]);
+                            split3_f16(v[q][nt].z * sc, h[0][2], h[1][2], h[2][2]);
+                            split3_f16(v[q][nt].w * sc, h[0][3], h[1][3], h[2][3]);
+                        } else {
+                            split3(v[q][nt].x, h[0][0], h[1][0], h[2][0]);
+                            split3(v[q][nt].y, h[0][1], h[1][1], h[2][1]);
+                            split3(v[q][nt].z, h[0][2], h[1][2], h[2][2]);
+                            split3(v[q][nt].w, h[0][3], h[1][3], h[2][3]);
+                        }
                         if constexpr (T::kQ2K) {
                             // sums of each 16 activations (four consecutive lanes hold them): [block][half][column]
                             float sum = (v[q][nt].x + v[q][nt].y) + (v[q][nt].z + v[q][nt].w);
@@ -1193,7 +1318,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
             }
         }
         const int64_t r0 = (int64_t)(rs - mat.rs_begin) * kStageRows;
-        if (r0 + 16 * warp < mat.rows) {
+        if (r0 + 16 * mt < mat.rows) {
             const uint32_t row = wrow + (uint32_t)slot * kStageBytes, wt = row + 4u * t;
             const uint32_t tab = smem_u32(smem + p.tab_off) + (uint32_t)warp * T::kTableBytes, tabg = tab + (uint32_t)kTabRow * g;
             const uint32_t sx = smem_u32(smem + p.sx_off) + (uint32_t)(8 * j) * kSxBlockBytes + 8u * t;
@@ -1228,6 +1353,19 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                     stage_q6k<NT, true>(wt + (o & ~3u), tabg, xp, y);
                 else
                     stage_q6k<NT, false>(wt + o, tabg, xp, y);
+            } else if constexpr (T::kF16) {
+                const uint32_t wr = wrow + (uint32_t)slot * kStageBytes;
+                if (warp < 8) {
+                    block_step_f16<NT, 0, 0>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 0, 1>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 1, 0>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 1, 1>(wr, sw, sx, xp, y);
+                } else {
+                    block_step_f16<NT, 2, 0>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 2, 1>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 3, 0>(wr, sw, sx, xp, y);
+                    block_step_f16<NT, 3, 1>(wr, sw, sx, xp, y);
+                }
             } else {
                 block_step<T, NT, 0, 0>(wt, row, tabg, sx, xp, y);
                 block_step<T, NT, 0, 1>(wt, row, tabg, sx, xp, y);
@@ -1914,25 +2052,33 @@ int launch_tc_columns(const MmaParams& p, const MmaMaps& maps, int grid, size_t 
         if (p.batch > 8) return launch_tc<T, 16>(p, maps, grid, smem_bytes, overlap, stream);
     return launch_tc<T, 8>(p, maps, grid, smem_bytes, overlap, stream);
 }
-// Which launches take the tcgen05 kernel.  f16: all.  Quantised formats: up to eight columns of q4_K, q4_0, q8_0 and four of
-// q4_1, when there are enough stages (256 rows x 256 columns) per SM: a stage is cheaper there, but the first one takes
-// about 1 us longer to get through (conversion with scales, decode -> tensor memory -> product -> read back, nothing of it
-// overlapped yet).  Measured, us, warp-level -> tcgen05, 3 or 4 | 8 columns:
-//   q4_K  28672 x 4096 (12.1 stages per SM) 29.3 -> 21.9 | 29.2 -> 25.4   8192 x 4096 (3.5) 11.4 -> 10.6 | 11.5 -> 12.0
-//   q4_0  28672 x 4096                      25.3 -> 22.2 | 25.2 -> 24.3   8192 x 4096       10.0 -> 10.4 | 10.2 -> 11.4
-//   q8_0  28672 x 4096                      30.4 -> 26.8 | 30.4 -> 28.9   8192 x 4096       11.8 -> 11.5 | 12.1 -> 12.8
-//   q4_1  28672 x 4096                      26.7 -> 22.0 | 26.6 -> 27.4   (its offsets are applied in fp32)
+// Which launches take the tcgen05 kernel.  A stage (256 rows x 256 columns, f16 128 x 256) is cheaper there, but the first one
+// takes longer to get through (conversion with scales, decode -> tensor memory -> product -> read back, nothing of it
+// overlapped yet), and so does each further run of a CTA's range.  Stages per SM decide.  Measured, us, warp-level ->
+// tcgen05, without | with launch overlap:
+//   f16  16 columns  2048 x 2048 (0.9 stages per SM) 9.1 -> 9.4 | 6.1 -> 6.6   4096 x 2048 (1.7) 12.8 -> 11.9 | 9.2 -> 8.9
+//         5 columns  2048 x 2048                     8.0 -> 8.2 | 4.9 -> 5.2   4096 x 2048       10.8 -> 10.2 | 7.3 -> 7.1
+//         3 columns   512 x 2048 (0.2)               7.3 -> 6.6 | 4.7 -> 4.7   4096 x 2048       10.8 -> 9.5 | 7.1 -> 6.6
+//   q4_K  8 columns  10752 x 4096 (4.5)            18.3 -> 18.7 | 14.5 -> 15.1  12288 x 4096 (5.2) 20.5 -> 19.3 | 17.1 -> 15.6
+//         3 columns   9472 x 4096 (4.0)            15.7 -> 14.0 | 13.2 -> 11.3  19200 x 4096 (8.1) 25.9 -> 20.6 | 22.6 -> 17.5
+//   q4_0  8 columns   6144 x 14336 (9.1)           24.2 -> 25.1 | 21.3 -> 22.3  28672 x 4096 (12.1) 29.2 -> 27.9 | 25.7 -> 24.6
+//         3 columns  10752 x 4096                  16.5 -> 16.4 | 12.4 -> 13.0  12288 x 4096       18.2 -> 17.0 | 15.0 -> 13.6
+//   q8_0  8 columns  16640 x 4096 (7.0)            23.6 -> 23.1 | 20.7 -> 20.2  14336 x 4096 (6.1) 21.8 -> 21.2 | 18.8 -> 19.0
+//         3 columns   9472 x 4096                  16.2 -> 15.2 | 13.5 -> 12.4
+//   q4_1  3 columns  10752 x 4096                  17.6 -> 16.5 | 13.2 -> 13.1;  at 8 columns 28672 x 4096 26.6 -> 27.4
+//                                                  (its offsets are applied in fp32)
 // q5_0, q5_1 and q5_K measured slower or equal (their fifth bits cost as much to place in either form); q6_K and q2_K have
 // scales per 16 weights and row pieces off the 16-byte grid; 9 to 16 columns spill (64 sums to read back per lane and stage).
 bool takes_tc(int fmt, int64_t n_stages, int batch) {
-    if (fmt == LW_F16) return true;
+    const bool few = batch <= 4;
     int per_sm;
     switch (fmt) {
-        case LW_Q4_K: per_sm = 4; break;
-        case LW_Q4_0:
-        case LW_Q8_0: per_sm = batch <= 4 ? 4 : 7; break;
+        case LW_F16: return few || n_stages > device_sm_count();
+        case LW_Q4_K: per_sm = few ? 4 : 5; break;
+        case LW_Q4_0: per_sm = few ? 5 : 10; break;
+        case LW_Q8_0: per_sm = few ? 4 : 7; break;
         case LW_Q4_1:
-            if (batch > 4) return false;
+            if (!few) return false;
             per_sm = 4;
             break;
         default: return false;
@@ -2021,8 +2167,9 @@ bool mma_plan(int fmt, bool tc, int64_t cols, int nt, int& chunk_cols, int& ring
     extra_bytes = fmt == LW_Q2_K ? (size_t)(1024 / 32) * 128 + (size_t)kMmaWarps * MmaQ2K::kTableBytes
                   : (fmt == LW_Q4_K || fmt == LW_Q5_K || fmt == LW_Q6_K)
                       ? (size_t)(1024 / 32) * kSxBlockBytes + (size_t)kMmaWarps * MmaQ4K::kTableBytes
-                      : ((fmt == LW_Q4_1 || fmt == LW_Q5_1) ? (size_t)(1024 / 32) * kSxBlockBytes : 0);
-    const size_t budget = kSmemPerCta - kMmaHeader - extra_bytes;
+                      : ((fmt == LW_F16 || fmt == LW_Q4_1 || fmt == LW_Q5_1) ? (size_t)(1024 / 32) * kSxBlockBytes : 0);
+    // (f16: up to 1 KB more goes into aligning the swizzled stages)
+    const size_t budget = kSmemPerCta - kMmaHeader - extra_bytes - (fmt == LW_F16 ? 1024 : 0);
     // the largest chunk that leaves room for two stages (q8_0, 458752 x 4096, 8 columns: 0.40 ms with chunks of
     // 1024 columns and two 68 KB stages against 0.49 ms with chunks of 256 and three)
     for (int kx = 1024; kx >= 256; kx /= 2) {
@@ -2180,6 +2327,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         case LW_Q4_K: return launch_tc_columns<TcK4>(p, maps, grid, smem_bytes, ov, stream);
     }
     switch (fmt) {
+        case LW_F16: return launch_mma_columns<MmaF16>(p, maps, grid, smem_bytes, ov, stream);
         case LW_Q8_0: return launch_mma_columns<MmaQ80>(p, maps, grid, smem_bytes, ov, stream);
         case LW_Q4_0: return launch_mma_columns<MmaQ40>(p, maps, grid, smem_bytes, ov, stream);
         case LW_Q4_1: return launch_mma_columns<MmaLegacy<LW_Q4_1>>(p, maps, grid, smem_bytes, ov, stream);

@@ -445,3 +445,22 @@ def test_matvec_batched_large_group_and_copy_that_never_comes():
     lw.matvec_group(lw.Q4_0, cols, items, batch=batch)
     torch.cuda.synchronize()
     assert lw.device_status() == 0
+
+
+# the two batched kernels for f16 on either side of their line (128-row stages x 256 columns: one per SM), from five columns
+# on; q4_0 and q4_K on either side of theirs (256-row stages: 10 resp. 5 per SM from five columns on, 5 for q4_0 below that)
+EITHER_SIDE = [(lw.F16, 128 * 148, 256, 5), (lw.F16, 128 * 148 + 1, 256, 5), (lw.F16, 2177, 2048, 8), (lw.F16, 2433, 2048, 16),
+               (lw.F16, 9, 512, 16), (lw.F16, 18945, 256, 9), (lw.Q4_K, 47104, 1024, 8), (lw.Q4_K, 47360, 1024, 8),
+               (lw.Q4_0, 94465, 1024, 5), (lw.Q4_0, 94720, 1024, 5), (lw.Q4_0, 47104, 1024, 3), (lw.Q4_0, 47360, 1024, 3)]
+
+
+@pytest.mark.parametrize("fmt,rows,cols,batch", EITHER_SIDE)
+def test_matvec_batched_on_either_side_of_the_kernels_line(fmt, rows, cols, batch):
+    n = min(rows, 500)
+    some = quantized_weights(fmt, n, cols, seed=75, tensor_id=fmt, outlier_p=0.01).reshape(n, -1)
+    pick = np.random.default_rng(75).integers(0, n, rows)
+    X = synth.activations(75, rows, batch, cols).reshape(batch, cols)
+    y_ref, s_ref = oracle.matvec(fmt, some, n, cols, X, batch, nthreads=4)
+    for overlap in (False, True):
+        y = gpu_matvec(fmt, np.ascontiguousarray(some[pick]), rows, cols, X, batch, overlap=overlap, repeat=2).reshape(batch, rows)
+        check_matvec(y, np.asarray(y_ref).reshape(batch, n)[:, pick], np.asarray(s_ref).reshape(batch, n)[:, pick], "fmt %d" % fmt)
