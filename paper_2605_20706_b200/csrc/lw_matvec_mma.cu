@@ -104,8 +104,9 @@ struct MmaParams {
     MmaItem item[kMmaMaxItems];
     int n_items;
     int total_rs;         // row stages of all matrices
-    int share, extra;     // stages of a CTA; the first `extra` CTAs take one more (64-bit divisions in every warp's prologue
-                          // cost 0.3 us)
+    // Stages of a CTA, and how many CTAs take one more: CTA b starts at share * b + min(b * extra_step >> 16, extra)
+    // (divisions in every warp's prologue cost 0.2-0.3 us).
+    int share, extra, extra_step;
     int spc_shift;        // log2 of the stages per (chunk, row stage)
     int batch;            // columns of this launch (<= 8 NT)
     int chunk_cols;       // 256, 512 or 1024: columns whose activations are resident at a time
@@ -1012,6 +1013,11 @@ __global__ void __launch_bounds__(256) zero_kernel(const __grid_constant__ ZeroL
     }
 }
 
+// First stage of a CTA.
+__device__ __forceinline__ unsigned first_stage(const MmaParams& p, unsigned cta) {
+    return (unsigned)p.share * cta + min(cta * (unsigned)p.extra_step >> 16, (unsigned)p.extra);
+}
+
 // Where a CTA is in its range of stages: chunk c, row stage rs (numbered through all matrices of the launch) of
 // matrix `it`, sub-stage j of the chunk, ring slot and the parity of the slot's current use.  Stepped without
 // divisions.
@@ -1065,8 +1071,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
     const uint32_t x_pitch = 2u * Kx + kXPad;                         // bytes between columns of a plane
     const uint32_t plane_pitch = NB * x_pitch;
     const int spc = 1 << p.spc_shift;                                 // stages per (chunk, row stage)
-    const unsigned first = (unsigned)p.share * blockIdx.x + min(blockIdx.x, (unsigned)p.extra);
-    const unsigned last = first + (unsigned)p.share + (blockIdx.x < (unsigned)p.extra ? 1u : 0u);
+    const unsigned first = first_stage(p, blockIdx.x), last = first_stage(p, blockIdx.x + 1);
     const int ring = p.ring;
 
     // With programmatic dependent launch this kernel may have been placed while its predecessor on the stream
@@ -1517,8 +1522,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
     const int Kx = p.chunk_cols;
     const uint32_t plane_bytes = (uint32_t)(Kx / 8) * kKGroup;
     const int spc = 1 << p.spc_shift;                                 // stages per (chunk, row stage)
-    const unsigned first = (unsigned)p.share * blockIdx.x + min(blockIdx.x, (unsigned)p.extra);
-    const int count = p.share + (blockIdx.x < (unsigned)p.extra ? 1 : 0);
+    const unsigned first = first_stage(p, blockIdx.x);
+    const int count = (int)(first_stage(p, blockIdx.x + 1) - first);
     const int ring = p.ring;
 
     // nothing of X or Y is touched before grid_dependency_wait() returns (see above)
@@ -2302,6 +2307,13 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
     if ((int64_t)grid > n_stages && !self_clear) grid = (int)n_stages;   // self-clearing: every SM, so launches never overlap
     p.share = (int)(n_stages / grid);
     p.extra = (int)(n_stages % grid);
+    // Which CTAs take the extra stages: spread evenly, or the first ones.  With few stages per CTA the first ones (more ranges
+    // start at even stages and lie in one run), with a handful of extra stages too, and for f16 with up to four columns;
+    // else spread.  us, first -> spread, with launch overlap: 4096 x 4096 (256 stages on 148 SMs) q5_1 5 columns 7.7 -> 8.3,
+    // 14336 x 4096 (896) 19.3 -> 19.7; 10752 x 4096 (672) q6_K 4 columns 16.3 -> 15.5, 32000 x 4096 (2000) 34.7 -> 33.7,
+    // q4_K 8 columns 28.2 -> 26.5; f16 14336 x 4096 (1792) 3 columns 24.9 -> 25.5, 8 columns 24.9 -> 23.8.
+    const bool lead = p.share < 4 || 16 * p.extra <= grid || (fmt == LW_F16 && batch <= 4);
+    p.extra_step = lead ? 65536 : (int)((65536ll * p.extra + grid - 1) / grid);
     p.spc_shift = p.chunk_cols == 1024 ? 2 : p.chunk_cols == 512 ? 1 : 0;
     p.drop_stage = -1;
     p.n_next = n_next;
