@@ -207,8 +207,8 @@ int lw_matvec(int fmt, const void* W_blocks, int64_t rows, int64_t cols, const f
         }
     } else if (batch == 1 && variant == LW_VARIANT_GENERIC && forced_variant() == LW_VARIANT_AUTO &&
                matvec_imma_supported(fmt, rows, cols)) {
-        // rows that no streaming kernel takes (no multiple of 16 bytes, or of 256 columns): 18 -> 9 us for q4_0 11007 x
-        // 2848, 63 -> 30 us for q6_K 32000 x 3072 against the generic kernel, which is left with rows wider than 16384
+        // rows that no streaming kernel takes (no multiple of 16 bytes, or of 256 columns); the generic kernel is left with
+        // narrow matrices and with rows wider than 16384
         err = launch_matvec_imma(fmt, W_blocks, rows, cols, X, Y, g_overlap.load() != 0, s);
     } else if (variant != LW_VARIANT_GENERIC && batch > 1)
         err = launch_matvec_stream_batched(fmt, W_blocks, rows, cols, X, Y, batch, g_overlap.load() != 0, s);

@@ -41,8 +41,8 @@ int launch_matvec_stream_group(int fmt, bool integer_dot, int64_t cols, int n_it
 // `counter` is a device word owned by the caller (cleared on the stream by the launch).
 bool matvec_sequence_supported(int fmt, int n_items, const lw_seq_item* items);
 int launch_matvec_sequence(int fmt, int n_items, const lw_seq_item* items, unsigned* counter, cudaStream_t stream);
-// Integer tensor-core kernel, batch 1 (lw_matvec_imma.cu): widths up to 16384 whose rows the streaming kernels do not
-// take (q4_K and q5_K have none).
+// Integer tensor-core kernel, batch 1 (lw_matvec_imma.cu): widths from about 1024 up to 16384 whose rows the streaming
+// kernels do not take (q4_K and q5_K have none).
 bool matvec_imma_supported(int fmt, int64_t rows, int64_t cols);
 int launch_matvec_imma(int fmt, const void* W, int64_t rows, int64_t cols, const float* X, float* Y, bool overlap,
                        cudaStream_t stream);

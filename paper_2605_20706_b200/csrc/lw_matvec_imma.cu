@@ -958,10 +958,17 @@ int launch_one(const ImmaParams& p, int grid, size_t smem_bytes, bool overlap, c
 
 }  // namespace
 
+// Narrow matrices stay with the generic kernel: its time grows with the width (a warp walks a row), this one's fixed part
+// is 3.5 us (2.8 under launch overlap).  us, generic -> this kernel, weights from memory: q4_0 1000 rows x 800 columns 3.9 ->
+// 3.8, x 1056 5.0 -> 3.9, x 2080 8.1 -> 4.1; 4096 x 800 4.5 -> 4.8, x 1056 5.4 -> 5.2; 11007 x 544 6.7 -> 7.2, x 800 8.3 ->
+// 7.3; q6_K 1000 x 768 3.7 -> 4.1, x 1280 5.1 -> 4.5, 11007 x 768 8.7 -> 8.0; q2_K, which the generic kernel decodes in whole
+// words, 4096 x 1280 4.9 -> 5.5, x 1792 6.2 -> 5.8, 11007 x 768 6.8 -> 7.5, x 1280 9.8 -> 9.3.
 bool matvec_imma_supported(int fmt, int64_t rows, int64_t cols) {
     ImmaParams p;
     size_t smem = 0;
-    return rows >= 1 && plan(fmt, rows, cols, 148, p, smem);
+    const int64_t least = fmt == LW_Q2_K ? 1536 : 1024;
+    const bool wide = cols >= least || (4 * cols >= 3 * least && rows >= 8192);
+    return rows >= 1 && wide && plan(fmt, rows, cols, 148, p, smem);
 }
 
 int launch_matvec_imma(int fmt, const void* W, int64_t rows, int64_t cols, const float* X, float* Y, bool overlap,

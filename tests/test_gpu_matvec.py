@@ -464,3 +464,20 @@ def test_matvec_batched_on_either_side_of_the_kernels_line(fmt, rows, cols, batc
     for overlap in (False, True):
         y = gpu_matvec(fmt, np.ascontiguousarray(some[pick]), rows, cols, X, batch, overlap=overlap, repeat=2).reshape(batch, rows)
         check_matvec(y, np.asarray(y_ref).reshape(batch, n)[:, pick], np.asarray(s_ref).reshape(batch, n)[:, pick], "fmt %d" % fmt)
+
+
+# widths off the grid on either side of the line between the generic and the integer kernel
+NARROW = [(f, r, c) for f in (lw.F16, lw.Q8_0, lw.Q4_0, lw.Q4_1, lw.Q5_0, lw.Q5_1)
+          for r, c in [(1, 1056), (150, 1056), (151, 992), (8191, 800), (8192, 800), (8200, 736)]]
+NARROW += [(lw.Q6_K, 8192, 768), (lw.Q6_K, 8191, 768), (lw.Q6_K, 3, 1280), (lw.Q2_K, 8192, 1280), (lw.Q2_K, 8191, 1280), (lw.Q2_K, 3, 1792)]
+
+
+@pytest.mark.parametrize("fmt,rows,cols", NARROW)
+def test_matvec_of_narrow_rows_off_the_grid(fmt, rows, cols):
+    n = min(rows, 400)
+    some = quantized_weights(fmt, n, cols, seed=63, tensor_id=fmt, outlier_p=0.01).reshape(n, -1)
+    pick = np.random.default_rng(63).integers(0, n, rows)
+    X = synth.activations(63, rows, 1, cols)
+    y_ref, s_ref = oracle.matvec(fmt, some, n, cols, X, 1, nthreads=4)
+    y = gpu_matvec(fmt, np.ascontiguousarray(some[pick]), rows, cols, X, overlap=True, repeat=2)
+    check_matvec(y, np.asarray(y_ref).reshape(1, n)[:, pick], np.asarray(s_ref).reshape(1, n)[:, pick], "fmt %d" % fmt)
