@@ -112,7 +112,7 @@ struct StreamParams {
 // and the younger one runs its last quarter alone at half the SM's throughput).
 // DROP builds the testing aid of lw_debug_drop_copy into the kernel (one copy is never requested); the kernels
 // that serve ordinary calls are built without it, so it costs them nothing.
-template <class T, int NG, bool DROP = false>
+template <class T, int NG, bool DROP = false, bool AHEAD = true>
 __global__ void __launch_bounds__(NG* kThreads, NG == 1 ? T::kMinCtas : 1)
     matvec_stream_kernel(const StreamParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(NG* kThreads, NG == 1 ? T::kMinCtas : 1)
     // already in the L2: 1B q4_0 335, 321, 317, 317, 318, 323; 8B q4_K 1273, 1258, 1251, 1247, 1248, 1253; 1B f16 562, 547,
     // 540, 527.  Activations not in the L2, 8B q4_K in a graph: 1234; 1234 (16 KB), 1246 (32 KB) with the rows alone, 1211
     // and 1216 with the activations in front.
-    if (tid == 0 && rows_here > 0) {
+    if (AHEAD && tid == 0 && rows_here > 0) {
         constexpr int64_t most = T::kIntegerDot ? 16 * 1024 : 32 * 1024;
         if (512 * (int64_t)cta < 4 * p.cols) l2_prefetch(Xm + 128 * cta, 512);       // (cols is a multiple of 256)
         const int64_t all = (int64_t)rows_here * row_bytes;
@@ -701,14 +701,14 @@ Plan make_plan(int fmt, bool integer_dot, int64_t rows, int64_t cols, int num_sm
     return pl;
 }
 
-template <class T, int NG, bool DROP = false>
+template <class T, int NG, bool DROP = false, bool AHEAD = true>
 int launch_groups(Plan& pl, bool overlap, cudaStream_t stream) {
     static bool attr_set[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(matvec_stream_kernel<T, NG, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(matvec_stream_kernel<T, NG, DROP, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemMaxCta);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
@@ -723,7 +723,7 @@ int launch_groups(Plan& pl, bool overlap, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, matvec_stream_kernel<T, NG, DROP>, pl.p);
+    return (int)cudaLaunchKernelEx(&cfg, matvec_stream_kernel<T, NG, DROP, AHEAD>, pl.p);
 }
 
 template <class T>
@@ -731,7 +731,12 @@ int launch_one(Plan& pl, bool overlap, cudaStream_t stream) {
     // the testing aid exists in one kernel only (q4_K, two worker groups)
     if constexpr (std::is_same<T, IdotQ4K>::value)
         if (pl.p.drop_unit >= 0 && pl.groups == 2) return launch_groups<T, 2, true>(pl, overlap, stream);
-    return pl.groups == 2 ? launch_groups<T, 2>(pl, overlap, stream) : launch_groups<T, 1>(pl, overlap, stream);
+    if (pl.groups != 2) return launch_groups<T, 1>(pl, overlap, stream);
+    // A launch that waits for nobody gains from the early L2 requests only where its CTAs have much to read (q4_K 4096 x 4096
+    // 5.65 -> 5.44 us, f16 4096 x 2048 6.3 -> 6.0); they cost 0.1-0.2 us where there is little (q5_1 1024 x 2048 3.59 -> 3.86) or
+    // the activations are a large part (q5_1 2048 x 8192 6.5 -> 6.9).
+    const bool much = (int64_t)pl.p.rows_per_cta * pl.p.row_bytes >= 40 * 1024 && (!T::kIntegerDot || pl.p.cols <= 4096);
+    return overlap || much ? launch_groups<T, 2>(pl, overlap, stream) : launch_groups<T, 2, false, false>(pl, overlap, stream);
 }
 
 // Plan for the batched kernel: one CTA per SM, `nb` columns of fixed-point activations resident.
