@@ -407,3 +407,50 @@ def test_a_copy_that_never_comes_in_the_integer_kernel(overlap):
     assert lw.device_status() == 0
     check_matvec(_run(fmt, blocks, rows, cols, X), y_ref, s_ref, "call after the fault")
     assert lw.device_status() == 0
+
+
+# launches that AUTO gives to the tcgen05 kernel: rows enough for its share per SM, made of a few hundred different ones
+LARGE_TC = [(lw.Q8_0, 9728, 4, 0.0), (lw.Q4_0, 12288, 4, 0.0), (lw.Q4_K, 12288, 8, 2.0 ** -18), (lw.Q4_1, 9728, 4, 2.0 ** -18),
+            (lw.F16, 200, 4, 2.0 ** -30), (lw.F16, 1500, 16, 2.0 ** -30)]
+
+
+@pytest.mark.parametrize("fmt,rows,batch,c_extra", LARGE_TC)
+def test_large_batched_launches_stay_inside_the_stated_bound(fmt, rows, batch, c_extra):
+    cols, n = 4096, 200
+    cols_x = []
+    for b in range(batch):
+        some, X = _adversarial(fmt, n, cols, seed=90 + fmt, zero_rest_of_vector=bool(b & 1))
+        cols_x.append(X[0] * (1.0 + b))
+    X = np.stack(cols_x).astype(np.float32)
+    some = some.reshape(n, -1)
+    pick = np.random.default_rng(76).integers(0, n, rows)
+    blocks = np.ascontiguousarray(some[pick])
+
+    def reference(X):
+        y_ref, s_ref = oracle.matvec(fmt, some.reshape(-1), n, cols, X, batch, nthreads=4)
+        e = np.concatenate([_extra_term(fmt, some.reshape(-1), n, cols, X[b:b + 1], c_extra) * np.ones((1, n)) for b in range(batch)])
+        return np.asarray(y_ref)[:, pick], np.asarray(s_ref)[:, pick], e[:, pick]
+
+    y_ref, s_ref, e = reference(X)
+    assert lw.query_variant(fmt, rows, cols, batch) == lw.VARIANT_MMA
+    y = _run(fmt, blocks, rows, cols, X, batch=batch)
+    worst = float((np.abs(y.astype(np.float64) - y_ref) / (RTOL * s_ref + ATOL + e)).max())
+    assert worst <= 1.0, "error / bound = %.3g" % worst
+    # a non-finite activation reaches every output of its column, and no other column
+    for bad in (np.nan, np.inf, -np.inf):
+        Xb = X.copy()
+        Xb[2, 100] = bad
+        y = _run(fmt, blocks, rows, cols, Xb, batch=batch)
+        assert not np.isfinite(y[2]).any() and np.isfinite(np.delete(y, 2, axis=0)).all()
+    # extreme magnitudes: alone, and an outlier beside ordinary activations, in columns of their own
+    Xe = np.zeros((batch, cols), np.float32)
+    Xe[0, 7] = 1e30
+    Xe[1, 9] = 1e-41
+    Xe[2, :] = 2.0 ** -100
+    Xe[3] = synth.activations(77, fmt, 1, cols)
+    Xe[3, 64] = 2.0 ** 40
+    y_ref, s_ref, e = reference(Xe)
+    y = _run(fmt, blocks, rows, cols, Xe, batch=batch)
+    finite = np.isfinite(y_ref.astype(np.float32))
+    assert (np.abs(y.astype(np.float64) - y_ref)[finite] <= (RTOL * s_ref + ATOL + e)[finite]).all()
+    assert lw.device_status() == 0
