@@ -7,13 +7,16 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "liblw.so")
-PYCALL = os.path.join(HERE, "_lwcall.so")          # CPython extension behind the binding's per-call functions
+# CPython extension behind the binding's per-call functions, named for the interpreter it is built for: another one does
+# not load it (the binding then makes those calls through ctypes)
+PYCALL = os.path.join(HERE, "_lwcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 SOURCES = ["lw_matvec_stream.cu", "lw_matvec_seq.cu", "lw_matvec_imma.cu", "lw_matvec_tile.cu", "lw_matvec_mma.cu", "lw_probe.cu", "lw_attn.cu", "lw_api.cu", "lw_hostpipe.cu", "lw_dequant.cu", "lw_matvec_generic.cu", "lw_quantize.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -27,29 +30,36 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PYCALL):
-        return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "lw.h"), __file__]
-    return any(os.path.getmtime(d) > t for d in deps)
+def _stale(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
 
 
 def _build_pycall() -> None:
-    import sysconfig
+    """Optional: without a C compiler or Python.h the binding works through ctypes, a few microseconds slower per call."""
     tmp = PYCALL + ".tmp.%d" % os.getpid()
-    proc = subprocess.run(["gcc", "-O2", "-std=c11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
-                           os.path.join(CSRC, "lw_pycall.c"), "-o", tmp], capture_output=True, text=True)
-    if proc.returncode != 0:
-        sys.stderr.write(proc.stdout + proc.stderr)
-        raise RuntimeError("gcc failed on lw_pycall.c")
+    try:
+        proc = subprocess.run(["gcc", "-O2", "-std=c11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                               os.path.join(CSRC, "lw_pycall.c"), "-o", tmp], capture_output=True, text=True)
+        failed = proc.stdout + proc.stderr if proc.returncode != 0 else None
+    except OSError as e:
+        failed = "gcc: %s" % e
+    if failed is not None:
+        sys.stderr.write("%s\nlw_pycall.c not built: calls from Python go through ctypes\n" % failed.rstrip())
+        return
     os.replace(tmp, PYCALL)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/*.cu + the host quantiser into liblw.so (no-op when up to date).  The translation
     units are compiled side by side (one nvcc process each) and linked at the end."""
-    if not force and not _stale():
+    source = os.path.join(CSRC, "lw_pycall.c")
+    untagged = os.path.join(HERE, "_lwcall.so")               # any interpreter would load it
+    if untagged != PYCALL and os.path.exists(untagged):
+        os.remove(untagged)
+    if force or _stale(PYCALL, [source, __file__]):
+        _build_pycall()
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "lw.h"), __file__]
+    if not force and not _stale(LIB, [d for d in deps if d != source]):
         return LIB
     import shutil
     import tempfile
@@ -79,7 +89,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(link.stdout + link.stderr)
             raise RuntimeError("nvcc failed linking liblw.so")
         os.replace(tmp, LIB)
-        _build_pycall()
     finally:
         shutil.rmtree(objdir, ignore_errors=True)
     return LIB

@@ -98,16 +98,42 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+class _CtypesCalls:
+    """The per-call entry points by ctypes, with the extension's arguments: for an interpreter it is not built for."""
+
+    @staticmethod
+    def matvec(fmt, W, rows, cols, X, Y, batch, stream):
+        return lib().lw_matvec(fmt, _addr(W), rows, cols, _addr(X), _addr(Y), batch, _stream_handle(stream))
+
+    @staticmethod
+    def dequant(fmt, W, n, out, stream):
+        return lib().lw_dequant(fmt, _addr(W), n, _addr(out), _stream_handle(stream))
+
+    @staticmethod
+    def sequence(fmt, n_items, items, workspace, workspace_bytes, stream):
+        return lib().lw_matvec_sequence(fmt, n_items, items, _addr(workspace), workspace_bytes, _stream_handle(stream))
+
+    @staticmethod
+    def sequence_batch(fmt, n_items, items, batch, stream):
+        return lib().lw_matvec_sequence_batch(fmt, n_items, items, batch, _stream_handle(stream))
+
+    @staticmethod
+    def attn_decode(fmt, K, V, q, out, n_head, n_kv_head, head_dim, n_pos, scale, workspace, workspace_bytes, stream):
+        return lib().lw_attn_decode(fmt, _addr(K), _addr(V), _addr(q), _addr(out), n_head, n_kv_head, head_dim, n_pos, scale,
+                                    _addr(workspace), workspace_bytes, _stream_handle(stream))
+
+
 def _calls():
-    """The extension module behind the per-call functions (csrc/lw_pycall.c), bound to the library on first use."""
+    """What makes the per-call functions' calls: the extension module (csrc/lw_pycall.c), bound to the library on first use,
+    or ctypes where there is none for this interpreter."""
     global _call
     if _call is None:
         L = lib()
         try:
             from . import _lwcall
-        except ImportError as e:
-            raise RuntimeError("_lwcall.so is missing beside liblw.so: build it with "
-                               "`python -m paper_2605_20706_b200.build`") from e
+        except ImportError:
+            _call = _CtypesCalls
+            return _call
         raw = device = None
         try:
             import torch

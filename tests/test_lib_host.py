@@ -294,3 +294,35 @@ def test_quantiser_of_zeros_of_either_sign_and_subnormals_gives_the_oracles_byte
     x[16:32] = rng.standard_normal((16, 32)) * 1e-38
     x[32:48] = np.abs(rng.standard_normal((16, 32))) * 1e-41
     np.testing.assert_array_equal(lw.quantize(fmt, x.reshape(-1)), oracle.quantize(fmt, x.reshape(-1)))
+
+
+def test_per_call_functions_without_the_extension(monkeypatch):
+    # the extension is named for the interpreter it is built for; where there is none for the running one, the same calls go
+    # through ctypes.  Errors found before any launch, with and without it.
+    import importlib.machinery
+    import sys
+    assert os.path.exists(lw_build.PYCALL)
+    assert lw_build.PYCALL.endswith(importlib.machinery.EXTENSION_SUFFIXES[0])
+    assert not os.path.exists(os.path.join(lw_build.HERE, "_lwcall.so"))
+    x = np.zeros(64, np.float32)
+
+    def codes():
+        out = []
+        for call in (lambda: lw.matvec(99, x, 1, 32, x, x, 1, 0), lambda: lw.matvec(lw.Q8_0, None, 1, 32, x, x, 1, 0),
+                     lambda: lw.matvec(lw.Q8_0, x, 1, 33, x, x, 1, 0), lambda: lw.matvec(lw.Q8_0, x, 1, 32, x, x, 17, 0),
+                     lambda: lw.dequant(lw.Q8_0, x, 33, x, 0), lambda: lw.matvec_sequence(lw.Q8_0, [(x, 1, 33, x, x, 0)], x, 0, 0),
+                     lambda: lw.matvec_sequence_batch(lw.Q8_0, [(x, 1, 33, x, x, 0)], 2, 0),
+                     lambda: lw.attn_decode(lw.Q4_K, x, x, x, x, 1, 1, 64, 1, 1.0, x, 0, 0)):
+            with pytest.raises(lw.LwError) as e:
+                call()
+            out.append((e.value.code, str(e.value)))
+        return out
+
+    monkeypatch.setattr(lw, "_call", None)
+    by_extension = codes()
+    assert lw._call.__name__.endswith("_lwcall")
+    monkeypatch.setattr(lw, "_call", None)
+    monkeypatch.setitem(sys.modules, "paper_2605_20706_b200._lwcall", None)       # an import that fails
+    monkeypatch.delattr(sys.modules["paper_2605_20706_b200"], "_lwcall", raising=False)
+    assert codes() == by_extension
+    assert lw._call is lw._CtypesCalls
