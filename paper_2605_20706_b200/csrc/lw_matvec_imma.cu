@@ -234,9 +234,7 @@ __device__ __forceinline__ void static_for(F f) {
 //   kChains           chains of four units (units: blocks of 32, or runs of 16 where the scales are per 16)
 //   kOffset           added to every code (exactly, through the initial accumulators)
 //   kHasMin           a weight has an additive term: the unit's sum of activations times `min`
-//   kHalfScale        the codes of odd units are fed in as 16 * code
 //   kMayStraddle      rows may start two bytes off the word grid
-//   kMayBeRagged      row pieces may start off the 16-byte grid
 //   rows<GEN, NO>()   products of NO groups of eight rows with the warp's 256 columns: per group the sums of rows 2 t
 //                     and 2 t + 1 over the lane's units.  r = the lane's row g with 4 t added; s0, s1 = addresses of rows
 //                     2 t and 2 t + 1; nlive = live blocks of the piece (the last piece of a
@@ -252,9 +250,7 @@ struct ImmaLegacy {
     static constexpr int kSuper = 8 * kBlock;
     static constexpr int kChains = 2, kGroup = 32;
     static constexpr int kOffset = FMT == LW_Q4_0 ? -8 : FMT == LW_Q5_0 ? -16 : 0;
-    static constexpr bool kHalfScale = false;
     static constexpr bool kMayStraddle = FMT == LW_Q4_0 || FMT == LW_Q5_0 || FMT == LW_Q8_0;
-    static constexpr bool kMayBeRagged = true;
     static constexpr bool kF16 = false;
 
     static __device__ __forceinline__ float weight(uint32_t row, int c) {
@@ -336,7 +332,7 @@ struct ImmaQ6K {
         const float dl = __fmul_rn(sh_half<208>(row), (float)sh_s8<192>(row + 8 * h + 2 * j + (l >> 4)));
         return __fmul_rn(dl, (float)((int)((lo & 15u) | (hi & 3u) << 4) - 32));
     }
-    static constexpr bool kHalfScale = false, kMayStraddle = true, kMayBeRagged = true;
+    static constexpr bool kMayStraddle = true;
     static constexpr bool kF16 = false;
 
     template <bool GEN, int NO>
@@ -401,7 +397,7 @@ struct ImmaQ2K {
         const float dl = __fmul_rn(sh_half<80>(row), (float)(pair & 15u)), ml = __fmul_rn(sh_half<82>(row), (float)(pair >> 4));
         return __fsub_rn(__fmul_rn(dl, (float)(q & 3u)), ml);
     }
-    static constexpr bool kHalfScale = false, kMayStraddle = false, kMayBeRagged = true;
+    static constexpr bool kMayStraddle = false;
     static constexpr bool kF16 = false;
 
     template <bool GEN, int NO>
@@ -605,8 +601,7 @@ __device__ __forceinline__ void load_x(XState<T::kChains>& x, uint32_t xb, uint3
             x.init[ch][0] = x.init[ch][1] = kIntMagic + T::kOffset * sum_lo;
             x.init[ch][2] = x.init[ch][3] = kIntMagic + T::kOffset * sum_hi;
         }
-        float d = __uint_as_float(sh32(meta));
-        if (T::kHalfScale && (s & 1)) d *= 0.0625f;
+        const float d = __uint_as_float(sh32(meta));
         x.klo[ch] = odd ? d * 256.f : d;
         x.khi[ch] = odd ? d * 16777216.f : d * 65536.f;
         x.nlo[ch] = -12582912.f * x.klo[ch];
@@ -820,7 +815,7 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                                 const uint32_t o8 = tile + (uint32_t)u * pitch + o * far;
                                 uint32_t rg = o8 + lane_g;
                                 R.s0[o] = o8 + lane_s, R.s1[o] = R.s0[o] + pitch;
-                                if (T::kMayBeRagged && ragged) {
+                                if (ragged) {
                                     rg += shift(u + o * step, g);
                                     R.s0[o] += shift(u + o * step, 2 * t), R.s1[o] += shift(u + o * step, 2 * t + 1);
                                 }

@@ -12,7 +12,7 @@
 //     rounded to eight: x1 + x2 = x (1 + e) with |e| <= 2^-16, so code * x1 + code * x2, accumulated in fp32 by the
 //     tensor core, is the product with the activation to 2^-16 relative -- 0.15 of the tolerance if every term of a
 //     row erred the same way, and an error that scales with |w x| term by term (an activation that meets a zero
-//     weight contributes exactly nothing).  Three terms (x exactly, -DLW_MMA_TERMS=3) measured 13 % slower at 8
+//     weight contributes exactly nothing).  Three terms (x exactly) measured 13 % slower at 8
 //     columns and 23 % at 16, where the tensor pipe binds.  A NaN or Inf stays non-finite (in x1 or x2).
 // The accuracy is that of the fp32 kernels' contract: |y - y_ref| <= 1e-4 * sum|w x| + 1e-6 with no extra term
 // (q4_0, q8_0; q4_K's sub-block offsets go onto fp32 sums of the activations and bring an extra term back, see MmaQ4K).
@@ -53,12 +53,8 @@
 namespace lw {
 namespace {
 
-#ifndef LW_MMA_WARPS
-#define LW_MMA_WARPS 16
-#endif
-constexpr int kMmaWarps = LW_MMA_WARPS;               // compute warps
-constexpr int kCtasPerSm = 16 / kMmaWarps;
-constexpr int kSmemPerCta = kCtasPerSm == 1 ? 227 * 1024 : 113 * 1024;
+constexpr int kMmaWarps = 16;                         // compute warps; one CTA per SM
+constexpr int kSmemPerCta = 227 * 1024;
 constexpr int kXR = 8 * 64 / (32 * kMmaWarps);        // quads per thread, piece and group of eight columns
 constexpr int kMmaComputeThreads = 32 * kMmaWarps;
 constexpr int kMmaThreads = kMmaComputeThreads + 32;  // plus the producer warp
@@ -68,10 +64,7 @@ constexpr int kStageUnits = kStageCols / 64;
 constexpr int kMaxRing = 4;
 constexpr int kXPad = 64;                             // bytes after each column of a plane: 16-byte loads of lanes
                                                       // (g, t) at 64 g + 16 t cover 128 distinct bytes per quarter warp
-#ifndef LW_MMA_TERMS
-#define LW_MMA_TERMS 2
-#endif
-constexpr int kTerms = LW_MMA_TERMS;                  // terms an activation is cut into (planes in shared memory)
+constexpr int kTerms = 2;                             // terms an activation is cut into (planes in shared memory)
 constexpr int kTabRow = 72;                           // bytes between rows of a warp's scale table: 64 of entries + 8, so the
                                                       // eight rows a warp reads at once (8-byte entries) fall into different banks
 constexpr int kSxBlockBytes = 64;                     // block sums of the activations: [block of 32][16 columns] floats
@@ -775,38 +768,22 @@ __device__ __forceinline__ void block_step(uint32_t wt, uint32_t row, uint32_t t
     }
 }
 
-// fp32 -> bf16 terms.  The first is x cut off after eight significant bits (exact difference).  With two terms
-// (the default) the second is the rest rounded to nearest: x1 + x2 = x (1 + e), |e| <= 2^-16.  With three
-// (-DLW_MMA_TERMS=3) the second is cut off as well and the third holds what is left: x1 + x2 + x3 == x exactly.
-// A NaN stays one (in x1, or in x2 when only its low payload bits were set); an Inf gives x2 = NaN.
-__device__ __forceinline__ void split3(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
+// fp32 -> two bf16 terms: x cut off after eight significant bits (exact difference) and the rest rounded to nearest:
+// x1 + x2 = x (1 + e), |e| <= 2^-16.  A NaN stays one (in x1, or in x2 when only its low payload bits were set); an Inf
+// gives x2 = NaN.
+__device__ __forceinline__ void split2(float x, uint32_t& h1, uint32_t& h2) {
     const uint32_t b1 = __float_as_uint(x) & 0xFFFF0000u;
-    const float r1 = x - __uint_as_float(b1);
-    h1 = b1 >> 16;
-    if (kTerms == 2) {
-        unsigned short r;
-        asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(r) : "f"(r1));
-        h2 = r;
-        h3 = 0;
-    } else {
-        const uint32_t b2 = __float_as_uint(r1) & 0xFFFF0000u;
-        const float r2 = r1 - __uint_as_float(b2);
-        h2 = b2 >> 16;
-        h3 = __float_as_uint(r2) >> 16;                 // at most eight significant bits are left: exact
-    }
+    unsigned short r;
+    asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(r) : "f"(x - __uint_as_float(b1)));
+    h1 = b1 >> 16, h2 = r;
 }
 
-// fp32 -> f16 terms of x (already scaled into the f16 range): cut off (exact differences) except the last, which
-// rounds the rest
-__device__ __forceinline__ void split3_f16(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
-    unsigned short a, b, c;
+// fp32 -> two f16 terms of x (already scaled into the f16 range), likewise
+__device__ __forceinline__ void split2_f16(float x, uint32_t& h1, uint32_t& h2) {
+    unsigned short a, b;
     asm("cvt.rz.f16.f32 %0, %1;" : "=h"(a) : "f"(x));
-    const float r1 = x - __half2float(__ushort_as_half(a));
-    if (kTerms == 2) asm("cvt.rn.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
-    else asm("cvt.rz.f16.f32 %0, %1;" : "=h"(b) : "f"(r1));
-    const float r2 = r1 - __half2float(__ushort_as_half(b));
-    asm("cvt.rn.f16.f32 %0, %1;" : "=h"(c) : "f"(r2));
-    h1 = a, h2 = b, h3 = c;
+    asm("cvt.rn.f16.f32 %0, %1;" : "=h"(b) : "f"(x - __half2float(__ushort_as_half(a))));
+    h1 = a, h2 = b;
 }
 
 // ------------------------------------------------------------------ tcgen05 kernel ---
@@ -1055,7 +1032,7 @@ struct Cursor {
 // DROP: a build for lw_debug_drop_copy (the producer requests nothing from stage p.drop_stage on, so the wait for
 // that stage runs out); the kernels of ordinary calls carry none of it.
 template <class T, int NT, bool DROP = false>
-__global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(const __grid_constant__ MmaParams p,
+__global__ void __launch_bounds__(kMmaThreads, 1) matvec_mma_kernel(const __grid_constant__ MmaParams p,
                                                                              const __grid_constant__ MmaMaps maps) {
     extern __shared__ __align__(128) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);               // [kMaxRing]
@@ -1262,7 +1239,7 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                     for (int nt = 0; nt < NT * kXR; ++nt) {
                         const int idx = tid + nt * kMmaComputeThreads;
                         const int b = idx >> 6, k4 = jj * (kStageCols / 4) + (idx & 63);
-                        uint32_t h[3][4];
+                        uint32_t h[kTerms][4];
                         if constexpr (T::kF16) {
                             // f16 terms of x * s, s = the power of two that brings the block's largest magnitude (eight
                             // consecutive lanes hold a block of 32) to 2^14 .. 2^15; 1 / s goes to [block][column]
@@ -1276,15 +1253,15 @@ __global__ void __launch_bounds__(kMmaThreads, kCtasPerSm) matvec_mma_kernel(con
                             if ((lane & 7) == 0)
                                 *reinterpret_cast<float*>(smem + p.sx_off + (size_t)(k4 >> 3) * kSxBlockBytes + 4 * b) =
                                     __uint_as_float((uint32_t)(254 - se) << 23);
-                            split3_f16(v[q][nt].x * sc, h[0][0], h[1][0], h[2][0]);
-                            split3_f16(v[q][nt].y * sc, h[0][1], h[1][1], h[2][1]);
-                            split3_f16(v[q][nt].z * sc, h[0][2], h[1][2], h[2][2]);
-                            split3_f16(v[q][nt].w * sc, h[0][3], h[1][3], h[2][3]);
+                            split2_f16(v[q][nt].x * sc, h[0][0], h[1][0]);
+                            split2_f16(v[q][nt].y * sc, h[0][1], h[1][1]);
+                            split2_f16(v[q][nt].z * sc, h[0][2], h[1][2]);
+                            split2_f16(v[q][nt].w * sc, h[0][3], h[1][3]);
                         } else {
-                            split3(v[q][nt].x, h[0][0], h[1][0], h[2][0]);
-                            split3(v[q][nt].y, h[0][1], h[1][1], h[2][1]);
-                            split3(v[q][nt].z, h[0][2], h[1][2], h[2][2]);
-                            split3(v[q][nt].w, h[0][3], h[1][3], h[2][3]);
+                            split2(v[q][nt].x, h[0][0], h[1][0]);
+                            split2(v[q][nt].y, h[0][1], h[1][1]);
+                            split2(v[q][nt].z, h[0][2], h[1][2]);
+                            split2(v[q][nt].w, h[0][3], h[1][3]);
                         }
                         if constexpr (T::kQ2K) {
                             // sums of each 16 activations (four consecutive lanes hold them): [block][half][column]
@@ -1981,22 +1958,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) matvec_tc_kernel(const __grid_c
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-template <class T, int NT, bool DROP = false>
-int launch_mma(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap,
-               cudaStream_t stream) {
-    // self-clearing launches are cooperative (their CTAs wait for one another) and ordinary in stream order
+template <auto kernel>
+int launch_batched(const MmaParams& p, const MmaMaps& maps, int threads, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
     static bool attr_set[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(matvec_mma_kernel<T, NT, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
         if (e != cudaSuccess) return (int)e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kMmaThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
     // (a cooperative launch that also carries the programmatic attribute works but measured slower than the
@@ -2011,9 +1986,13 @@ int launch_mma(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_by
     }
     cfg.attrs = attr;
     cfg.numAttrs = (p.self_clear || overlap) ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, matvec_mma_kernel<T, NT, DROP>, p, maps);
+    return (int)cudaLaunchKernelEx(&cfg, kernel, p, maps);
 }
 
+template <class T, int NT, bool DROP = false>
+int launch_mma(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
+    return launch_batched<matvec_mma_kernel<T, NT, DROP>>(p, maps, kMmaThreads, grid, smem_bytes, overlap, stream);
+}
 template <class T>
 int launch_mma_columns(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
     return p.batch <= 8 ? launch_mma<T, 1>(p, maps, grid, smem_bytes, overlap, stream)
@@ -2022,31 +2001,7 @@ int launch_mma_columns(const MmaParams& p, const MmaMaps& maps, int grid, size_t
 
 template <class T, int CB, bool DROP = false>
 int launch_tc(const MmaParams& p, const MmaMaps& maps, int grid, size_t smem_bytes, bool overlap, cudaStream_t stream) {
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return (int)e;
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(matvec_tc_kernel<T, CB, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
-        if (e != cudaSuccess) return (int)e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = smem_bytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    if (p.self_clear) {
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-    } else {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = (p.self_clear || overlap) ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, matvec_tc_kernel<T, CB, DROP>, p, maps);
+    return launch_batched<matvec_tc_kernel<T, CB, DROP>>(p, maps, kTcThreads, grid, smem_bytes, overlap, stream);
 }
 
 // A launch holds 4, 8 or 16 columns (fewer accumulator columns to read back).
@@ -2239,7 +2194,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
         int cc = 0, rg = 0;
         size_t xb = 0, sb = 0, eb = 0;
         if (!mma_plan(fmt, tc, cols, nt, cc, rg, xb, sb, eb)) return (int)cudaErrorInvalidValue;
-        if (2 * ((kMmaHeader + xb + eb + 127) / 128 * 128 + (size_t)rg * sb + 1024) <= 228 * 1024 || kCtasPerSm != 1)   // (f16's alignment slack only adds)
+        if (2 * ((kMmaHeader + xb + eb + 127) / 128 * 128 + (size_t)rg * sb + 1024) <= 228 * 1024)   // (f16's alignment slack only adds)
             self_clear = false;
     }
     unsigned* grid_bar = nullptr;
@@ -2303,7 +2258,7 @@ int launch_matvec_mma_group(int fmt, int64_t cols, int n_items, const void* cons
     const size_t w_align = fmt == LW_F16 ? 1024 : 128;
     p.w_off = (uint32_t)((kMmaHeader + x_bytes + extra_bytes + w_align - 1) / w_align * w_align);
     const size_t smem_bytes = p.w_off + (size_t)p.ring * stage_bytes;
-    int grid = kCtasPerSm * device_sm_count();
+    int grid = device_sm_count();
     if ((int64_t)grid > n_stages && !self_clear) grid = (int)n_stages;   // self-clearing: every SM, so launches never overlap
     p.share = (int)(n_stages / grid);
     p.extra = (int)(n_stages % grid);
