@@ -137,6 +137,12 @@ __device__ __forceinline__ uint32_t sh_u8(uint32_t a) {
     asm volatile("ld.shared.u8 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
     return v;
 }
+template <int OFF>
+__device__ __forceinline__ uint32_t sh_u16(uint32_t a) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(v) : "r"(a), "n"(OFF));
+    return v;
+}
 __device__ __forceinline__ uint4 sh128(uint32_t a) {
     uint4 v;
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
@@ -253,16 +259,30 @@ struct ImmaLegacy {
     static constexpr bool kMayStraddle = FMT == LW_Q4_0 || FMT == LW_Q5_0 || FMT == LW_Q8_0;
     static constexpr bool kF16 = false;
 
-    static __device__ __forceinline__ float weight(uint32_t row, int c) {
-        const uint32_t b = row + (uint32_t)(c >> 5) * kBlock;
+    // sum of weight * X[c] over the columns c of block k whose bits are set in `word`
+    static __device__ __forceinline__ float sum_of(uint32_t row, int k, uint32_t word, const float* X) {
+        const uint32_t b = row + (uint32_t)k * kBlock;
         const float d = sh_half<0>(b);
-        if constexpr (kEight) return __fmul_rn((float)sh_s8<2>(b + (c & 31)), d);
-        const uint32_t nib = sh_u8<2 + (kHasMin ? 2 : 0) + (kFive ? 4 : 0)>(b + (c & 15));
-        int q = (int)(c & 16 ? nib >> 4 : nib & 15u);
-        if constexpr (kFive) q |= (int)((sh_u8<2 + (kHasMin ? 2 : 0)>(b + ((c & 31) >> 3)) >> (c & 7)) & 1u) << 4;
-        if constexpr (kHasMin) return __fadd_rn(__fmul_rn(d, (float)q), sh_half<2>(b));
-        return __fmul_rn((float)(q + kOffset), d);
+        float m = 0.f, sum = 0.f;
+        uint32_t five = 0;
+        if constexpr (kHasMin) m = sh_half<2>(b);
+        if constexpr (kFive) five = sh_u16<2 + (kHasMin ? 2 : 0)>(b) | sh_u16<4 + (kHasMin ? 2 : 0)>(b) << 16;
+#pragma unroll 2
+        for (; word != 0; word &= word - 1) {
+            const int c = __ffs((int)word) - 1;
+            float w;
+            if constexpr (kEight) {
+                w = __fmul_rn((float)sh_s8<2>(b + c), d);
+            } else {
+                const uint32_t nib = sh_u8<2 + (kHasMin ? 2 : 0) + (kFive ? 4 : 0)>(b + (c & 15));
+                const int q = (int)((nib >> (c >> 4 << 2) & 15u) | (five >> c & 1u) << 4);
+                w = kHasMin ? __fadd_rn(__fmul_rn(d, (float)q), m) : __fmul_rn((float)(q + kOffset), d);
+            }
+            sum = fmaf(w, X[c], sum);
+        }
+        return sum;
     }
+
     template <bool GEN, int J>
     static __device__ __forceinline__ void codes(const RowAddr& r, int t, uint32_t& b0, uint32_t& b1) {
         constexpr int B = J * kBlock;
@@ -326,11 +346,18 @@ __device__ __forceinline__ float uint_float23(uint32_t v) { return __uint_as_flo
 struct ImmaQ6K {
     static constexpr bool kHasMin = false;
     static constexpr int kSuper = 210, kChains = 4, kGroup = 16, kOffset = -32;
-    static __device__ __forceinline__ float weight(uint32_t row, int c) {
-        const int h = c >> 7, j = (c >> 5) & 3, l = c & 31;
-        const uint32_t lo = sh_u8<0>(row + 64 * h + l + 32 * (j & 1)) >> (j & 2 ? 4 : 0), hi = sh_u8<128>(row + 32 * h + l) >> (2 * j);
-        const float dl = __fmul_rn(sh_half<208>(row), (float)sh_s8<192>(row + 8 * h + 2 * j + (l >> 4)));
-        return __fmul_rn(dl, (float)((int)((lo & 15u) | (hi & 3u) << 4) - 32));
+    static __device__ __forceinline__ float sum_of(uint32_t row, int k, uint32_t word, const float* X) {
+        const int h = k >> 2, j = k & 3;
+        const uint32_t ql = row + 64 * h + 32 * (j & 1), qh = row + 32 * h, sc = row + 8 * h + 2 * j;
+        const float d = sh_half<208>(row), d0 = __fmul_rn(d, (float)sh_s8<192>(sc)), d1 = __fmul_rn(d, (float)sh_s8<193>(sc));
+        float sum = 0.f;
+#pragma unroll 2
+        for (; word != 0; word &= word - 1) {
+            const int l = __ffs((int)word) - 1;
+            const uint32_t q = (sh_u8<0>(ql + l) >> (j & 2 ? 4 : 0) & 15u) | (sh_u8<128>(qh + l) >> (2 * j) & 3u) << 4;
+            sum = fmaf(__fmul_rn(l < 16 ? d0 : d1, (float)((int)q - 32)), X[l], sum);
+        }
+        return sum;
     }
     static constexpr bool kMayStraddle = true;
     static constexpr bool kF16 = false;
@@ -391,11 +418,20 @@ struct ImmaQ6K {
 struct ImmaQ2K {
     static constexpr bool kHasMin = true;
     static constexpr int kSuper = 84, kChains = 4, kGroup = 16, kOffset = 0;
-    static __device__ __forceinline__ float weight(uint32_t row, int c) {
-        const int h = c >> 7, j = (c >> 5) & 3, l = c & 31;
-        const uint32_t pair = sh_u8<0>(row + 8 * h + 2 * j + (l >> 4)), q = sh_u8<16>(row + 32 * h + l) >> (2 * j);
-        const float dl = __fmul_rn(sh_half<80>(row), (float)(pair & 15u)), ml = __fmul_rn(sh_half<82>(row), (float)(pair >> 4));
-        return __fsub_rn(__fmul_rn(dl, (float)(q & 3u)), ml);
+    static __device__ __forceinline__ float sum_of(uint32_t row, int k, uint32_t word, const float* X) {
+        const int h = k >> 2, j = k & 3;
+        const uint32_t codes = row + 32 * h, p0 = sh_u8<0>(row + 8 * h + 2 * j), p1 = sh_u8<1>(row + 8 * h + 2 * j);
+        const float d = sh_half<80>(row), dmin = sh_half<82>(row);
+        const float d0 = __fmul_rn(d, (float)(p0 & 15u)), m0 = __fmul_rn(dmin, (float)(p0 >> 4));
+        const float d1 = __fmul_rn(d, (float)(p1 & 15u)), m1 = __fmul_rn(dmin, (float)(p1 >> 4));
+        float sum = 0.f;
+#pragma unroll 2
+        for (; word != 0; word &= word - 1) {
+            const int l = __ffs((int)word) - 1;
+            const float q = (float)(sh_u8<16>(codes + l) >> (2 * j) & 3u);
+            sum = fmaf(__fsub_rn(__fmul_rn(l < 16 ? d0 : d1, q), l < 16 ? m0 : m1), X[l], sum);
+        }
+        return sum;
     }
     static constexpr bool kMayStraddle = false;
     static constexpr bool kF16 = false;
@@ -530,28 +566,34 @@ __device__ __forceinline__ bool convert_x(const float* X, int cols, int padded, 
     return any;
 }
 
-// Adds weight * activation of the columns of a 256-column piece that are kept apart (bit table at `bits`, activations at X),
-// in fp32, to the row sums of a tile of n rows that the warp has just put into its table.  Eight rows at a time; the four
-// lanes of a row take the words of the bit table in turn.  `piece` = where the tile's row 0 has the piece in shared memory,
-// `at` = the table's entry of row 0, `shift0` = row 0's offset behind the boundary its copy started at, `rb` = what the next
-// row's offset differs by.
+// Adds weight * activation of the columns of a 256-column piece that are kept apart (bit table at `bits`, of whose eight words
+// those in `words` are not zero; activations at X), in fp32, to the row sums of a tile of n rows that the warp has just put
+// into its table.  Four groups of eight rows (from `first` on, `step` apart) at a time with a lane per row, or, with more than
+// two words or fewer rows, one group with four lanes per row that take the words in turn.  `piece` = where the tile's row 0 has
+// the piece in shared memory, `at` = the table's entry of row 0, `shift0` = row 0's offset behind the boundary its copy
+// started at, `rb` = what the next row's offset differs by.
 template <class T>
 __device__ __noinline__ void add_apart(uint32_t piece, uint32_t pitch, uint32_t shift0, uint32_t rb, uint32_t at, uint32_t bits,
-                                       const float* X, int n, int first, int step, int lane) {
+                                       uint32_t words, const float* X, int n, int first, int step, int lane) {
     __syncwarp();
-    for (int u = first; u < n; u += step) {
-        const int i = u + (lane >> 2);
+    const bool wide = __popc(words) <= 2 && n > first + step;
+    uint32_t mine = words;
+    if (!wide) mine = words & (0x11u << (lane & 3));
+    const int g = wide ? lane & 7 : lane >> 2;
+    for (int u = first + (wide ? (lane >> 3) * step : 0); __any_sync(0xFFFFFFFFu, u < n); u += wide ? 4 * step : step) {
+        const int i = min(u + g, n - 1);
         const uint32_t row = piece + (uint32_t)i * pitch + ((shift0 + (uint32_t)i * rb) & 15u);
         float sum = 0.f;
-        for (int k = lane & 3; k < 8; k += 4)
-            for (uint32_t word = sh32(bits + 4u * k); word != 0; word &= word - 1) {
-                const int c = 32 * k + __ffs((int)word) - 1;
-                sum = fmaf(T::weight(row, c), X[c], sum);
-            }
+        for (uint32_t m = mine; m != 0; m &= m - 1) {
+            const int k = __ffs((int)m) - 1;
+            sum += T::sum_of(row, k, sh32(bits + 4u * k), X + 32 * k);
+        }
         __syncwarp();
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
-        put_sum(at + (uint32_t)u * (4 * kComputeWarps) + 4u * (lane >> 2), sum, (lane & 3) == 0, true);
+        if (!wide) {
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+        }
+        put_sum(at + (uint32_t)u * (4 * kComputeWarps) + 4u * g, sum, u < n && (wide || (lane & 3) == 0), true);
     }
 }
 
@@ -745,7 +787,7 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
     const uint32_t lane_g = (uint32_t)g * pitch + (uint32_t)cw * T::kSuper, lane_s = (uint32_t)(2 * t) * pitch + (uint32_t)cw * T::kSuper;
     const bool straddle = ragged || (((uint32_t)cw * T::kSuper) & 2u);
     XState<T::kChains> x;
-    bool piece_apart = false;                        // are there any in this warp's 256 columns?
+    uint32_t words_apart = 0;                        // which of the eight words of this warp's 256 columns have any
     f2 xf[4];                                        // f16: the lane's eight activations
     for (int r0 = v0; r0 < v1; r0 += fold_rows) {
         const int r1 = min(v1, r0 + fold_rows);
@@ -762,7 +804,7 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                     xf[0] = pack2u(a.x, a.y), xf[1] = pack2u(a.z, a.w), xf[2] = pack2u(b.x, b.y), xf[3] = pack2u(b.z, b.w);
                 } else {
                     load_x<T>(x, xs + (uint32_t)(8 * sb) * kXBlock, base + kZeros, g, t);
-                    piece_apart = apart && __any_sync(0xFFFFFFFFu, sh32(base + kApartBits + 32u * sb + 4u * (lane & 7)) != 0);
+                    if (apart) words_apart = __ballot_sync(0xFFFFFFFFu, lane < 8 && sh32(base + kApartBits + 32u * sb + 4u * (lane & 7)) != 0);
                 }
             }
             const uint32_t coff = (uint32_t)c * chunk_sb * T::kSuper;
@@ -851,9 +893,9 @@ __global__ void __launch_bounds__(kImmaThreads, 1) matvec_imma_kernel(const __gr
                         int u = 8 * rgrp;
                         for (; u + step < n; u += 2 * step) products(std::integral_constant<int, 2>{}, u);
                         if (u < n) products(std::integral_constant<int, 1>{}, u);
-                        if (piece_apart)
+                        if (words_apart != 0)
                             add_apart<T>(tile + (uint32_t)cw * T::kSuper, pitch, ragged ? (uint32_t)r * rb + coff : 0u, ragged ? rb : 0u,
-                                         tab - 4u * (2 * t + (g & 1)), base + kApartBits + 32u * sb, p.X + 256 * sb, n, 8 * rgrp, step, lane);
+                                         tab - 4u * (2 * t + (g & 1)), base + kApartBits + 32u * sb, words_apart, p.X + 256 * sb, n, 8 * rgrp, step, lane);
                     }
                 }
                 __syncwarp();
