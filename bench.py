@@ -55,14 +55,14 @@ def arithmetic_of(fmt, batch):
     """What the kernels compute in (the `dtype` key): not a precision claim, the arithmetic that runs."""
     if fmt == "f16" and batch >= 3:
         return ("f32 in/out; f16 weights x two-term f16 split of the block-scaled fp32 activations on the tensor cores "
-                "(mma m16n8k16), fp32 accumulation")
+                "(mma m16n8k16, tcgen05.mma for larger launches), fp32 accumulation")
     if fmt == "f16":
         return "f32 in/out; f16 weights widened, fp32 FMA"
     if batch == 1:
         return "f32 in/out; activations as 24-bit block fixed point, int32 dp4a sums, fp32 block scales"
     if fmt in MMA_FORMATS and batch >= 3:
         return ("f32 in/out; exact bf16 weight codes x two-term bf16 split (16 significant bits) of the fp32 activations on the tensor cores "
-                "(mma m16n8k16), fp32 accumulation and block scales")
+                "(mma m16n8k16; larger launches of q4_K, q4_0, q4_1, q8_0: tcgen05.mma), fp32 accumulation and block scales")
     return "f32 in/out; batch > 1: per-column passes of the batch-1 kernel (24-bit block fixed point, int32 dp4a) or fp32 FMA tiles"
 
 

@@ -2,18 +2,18 @@
 // and q2_K at most widths), widths that are no multiple of 256 columns [paper Sec 3.2: the decode-phase mat-vec; Sec 3.3:
 // one decode routine per block format spliced into a common skeleton, weights decoded straight into registers].
 //
-// What bounds it: instructions (about 160 warp instructions per 2048 4-bit weights, 300 for q6_K, at 55-60 % of the
-// issue slots).  The generic kernel it took over from decodes from global memory in 2- and 4-byte loads: q6_K
-// 32000 x 3072 63 -> 30 us, q4_0 11007 x 2848 18 -> 9.3 us (back to back from Python 10.6).
+// What bounds it: instructions (217 warp instructions per 2048 weights of q4_0 at 88000 x 2848, prologue included, 377 of
+// q6_K at 64000 x 3072, at 57-59 % of the issue slots; HBM at a third), and on small matrices 3.5 us until the first tile's
+// products.  Against the generic kernel, which decodes from global memory in 2- and 4-byte loads: q6_K 32000 x 3072 63 ->
+// 31 us, q4_0 11007 x 2848 20.5 -> 9.5 (matvec_imma_supported has the line between the two).
 //
 // Arithmetic.  The activations of a block of 32 (16 where the format's scales are per 16) become fixed point relative
 // to the block's largest M: v = rint(x / d), |v| < 2^31, d a power of two, so that every element down to 2^-6 M is
 // represented exactly and one of 2^-17 M to 2^-14 of itself.  What does not fit -- smaller elements beside a large one,
 // magnitudes of 2^96 and more, Inf and NaN -- counts as zero there and is multiplied in fp32 with its exactly decoded
-// weight: every element keeps a relative accuracy of its own, whatever stands beside it.  One element in 60 000 of normally
-// distributed activations is kept apart like this.
-// v is written as four signed digits of base 256.  mma.m16n8k32 (s8 x u8 / s8 -> s32)
-// multiplies A (16 x 32) = digits of the activations with B (32 x 8) = the codes of one block of 8 weight rows:
+// weight: every element keeps a relative accuracy of its own, whatever stands beside it.  One element in 80 000 of normally
+// distributed activations is kept apart like this.  v is written as four signed digits of base 256.  mma.m16n8k32 (s8 x u8 /
+// s8 -> s32) multiplies A (16 x 32) = digits of the activations with B (32 x 8) = the codes of one block of 8 weight rows:
 //   A row m = g     : digit (g & 1)     of block s = g / 2 of the chain of four blocks,  g = 0..7
 //   A row m = g + 8 : digit 2 + (g & 1) of the same block
 // and zero in the rows of the other three blocks, so that four products accumulate into ONE set of accumulators
@@ -23,9 +23,10 @@
 // an offset of its own (q4_1, q5_1, q2_K), scale * sum of code * digit and offset * sum of digits nearly cancel when a large
 // activation meets a weight next to zero: they are added per digit, with one rounding.
 //
-// Work and data.  One CTA per SM: 16 compute warps and one copy warp.  The rows are cut evenly over the CTAs.  The copy warps bring tiles of rows into a ring of slots with 16-byte cp.async (rows
-// lie an odd multiple of 16 bytes apart in a slot, so the eight rows a warp reads at once fall into different banks;
-// 1-D bulk copies cannot pad, tiled bulk copies need row lengths that are multiples of 16, which odd widths have not).
+// Work and data.  One CTA per SM: 16 compute warps and one copy warp.  The rows are cut evenly over the CTAs.  The copy warp
+// brings tiles of rows into a ring of slots, one 1-D bulk copy per row, from the 16-byte boundary below the row to the one
+// above it where rows are off that grid (tiled bulk copies need row lengths that are multiples of 16).  Rows lie an odd
+// multiple of 16 bytes apart in a slot, so the eight rows a warp reads at once fall into different banks.
 // A compute warp owns one 256-column piece of the row (its A operands stay in registers, 32 of them) and walks the
 // tile's groups of eight rows; its row sums go to a table in shared memory that is folded once per 128 rows.
 //

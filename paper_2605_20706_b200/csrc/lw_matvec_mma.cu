@@ -799,8 +799,9 @@ __device__ __forceinline__ void split2_f16(float x, uint32_t& h1, uint32_t& h2) 
 // 0x000F000F gives two nibbles ready to multiply, 0x00F000F0 two nibbles times 16, and one packed addition takes q4_0's
 // 8 or q8_0's 128 off.  Up to 8 columns about 210 warp instructions per 2048 4-bit weights (decode and stores to tensor
 // memory 80, reading the sums back and scaling 55, the rest waits and loop), against 257 for the warp-level form (one
-// byte permute and one subtraction per pair of weights, fragments of two rows per lane, scale tables): that is the bound,
-// 56 % of the issue slots; the tensor pipe is busy a fifth of the time.
+// byte permute and one subtraction per pair of weights, fragments of two rows per lane, scale tables).  They fill 47 % of the
+// issue slots (57344 x 4096 q4_K, 8 columns), the tensor pipe is busy 15 % of the time: what bounds it is the latency of the
+// hand-over (store, wait, product, commit, load), which the four warpgroups cover in part.
 //
 // B: bf16 terms of x * s, s the power of two that brings the largest magnitude of 128 columns to 2^126..2^127, which with the
 // 2^-133 of the codes leaves products in the middle of fp32's range: no term is lost down to 2^-120 of the largest, and the
